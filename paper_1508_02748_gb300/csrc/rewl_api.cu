@@ -449,7 +449,7 @@ int create_impl(const rewl_config *cfg, const uint8_t *host_init_spins, void *d_
     // memory when a warp's share stays small, else global memory
     if (cfg->table_mode == REWL_TABLES_STAGED) p.smt = 1;
     else if (cfg->table_mode == REWL_TABLES_GLOBAL) p.smt = 0;
-    else p.smt = tree_smem_per_warp(p, true) * (size_t)(32 / p.group) <= 100 * 1024 ? 1 : 0;
+    else p.smt = tree_smem_per_warp(p, true, p.group) * (size_t)(32 / p.group) <= 100 * 1024 ? 1 : 0;
     if (p.sampler != REWL_SAMPLER_WARP) p.smt = 0;
     h->first_active = -1;
     for (int win = 0; win < d.nwin && h->first_active < 0; ++win)

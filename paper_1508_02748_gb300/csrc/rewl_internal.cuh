@@ -137,7 +137,7 @@ cudaError_t launch_sweep(const Params &p, uint64_t ntrials, int walkers_per_bloc
 // Sweep of walker w alone: one thread of the one-thread-per-walker kernel.
 cudaError_t launch_sweep_walker(const Params &p, int w, uint64_t ntrials, cudaStream_t s);
 cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int warps, bool smt, cudaStream_t s);
-size_t tree_smem_per_warp(const Params &p, bool smt);
+size_t tree_smem_per_warp(const Params &p, bool smt, int group);
 cudaError_t launch_exchange(const Params &p, int max_pairs, cudaStream_t s);
 cudaError_t launch_flat(const Params &p, cudaStream_t s);
 cudaError_t launch_decide(const Params &p, int flags, cudaStream_t s);

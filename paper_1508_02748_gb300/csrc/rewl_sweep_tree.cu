@@ -9,28 +9,31 @@
 // h = l + 1 - 2^d (bit k of h = outcome assumed for trial t+k).
 //
 // Per step every lane
-//   1. reads its trial's ring entry and the five spins around its site from
-//      the committed lattice, corrected for the sites its history flips: the
-//      ring entry carries, for each earlier trial of the step, which of the
-//      five positions that trial's site is (a one-hot code made when the
-//      ring was filled), so the correction is one mask and a fold;
-//   2. takes the moves of the earlier trials of its history by shuffle from
-//      the lanes that evaluated them and adds them up: its position (E, M)
-//      and the positions after each earlier trial;
-//   3. decides its own trial (Eq. 1) from the values the sequential chain
-//      sees there, ln g(b) = base(b) + (H(b) + visits earlier in the step)
-//      ln f.
+//   1. takes its trial from the ring and the five spins around its site from
+//      the committed lattice, corrected for the sites its history flips, and
+//      so has its trial's move;
+//   2. takes the moves of the accepted trials of its history by shuffle, the
+//      latest first, and adds them up: the position before and after its own
+//      trial.  A bin the path was in 2 accepted trials ago is the current one
+//      again iff the two moves cancel, so three sums say which bins were met
+//      before, and how often is a constant of the lane's history;
+//   3. reads the proposed bin's screen and visits and decides its own trial
+//      (Eq. 1) from the values the sequential chain sees there, ln g(b) =
+//      base(b) + (H(b) + visits earlier in the step) ln f.  The current bin
+//      needs no read: it is the bin the last accepted trial of the history
+//      proposed (a shuffle), or the step's first bin, which the lane without a
+//      node (G-1) reads.
 // One ballot gives the true path from the root: a lane is on it iff the
-// ballot bits of its ancestors are the outcomes its history assumes.  Lane k
-// of the path knows how often its bin was visited on the path up to trial
-// t+k (its own history's count plus one), so it writes that bin's H as the
-// count it had plus those visits; the lanes write in path order (one store
-// per depth, warp barriers between), so a bin visited again later ends with
-// the larger count.  The leaf posts the final position, its visits on the
-// path, its H and its screen value in a per-walker mailbox in shared memory
-// (a register lattice also gets the path's flipped sites there), so the
-// group adopts its new state without comparing the path's bins or reading
-// the table again.
+// ballot bits of its ancestors are the outcomes its history assumes.  The
+// path's last lane hands the new position and the path's outcomes round by
+// shuffle.  Each on-path lane that accepts writes the visits of the bin it
+// enters: the count it read, the path's earlier visits of that bin, and the
+// trials until the path leaves it, all known to it; a bin entered twice is
+// written in path order (few ordered stores).
+//
+// Nothing in a step branches by lane, and all groups of a warp step together:
+// collectives over part of a warp, and lanes that branch, run the groups of a
+// warp one after the other.
 //
 // Tables (exact formats only; REWL_F32 runs on the thread sampler): ln g(b)
 // = base(b) + max(H(b), 0) ln f, the base fixed during an iteration, so a
@@ -38,9 +41,9 @@
 // decision is screened in float from a 32-bit screen per bin, S(b) =
 // base(b) - c_w rounded to nearest (c_w one constant per walker, which
 // cancels in the difference and keeps the screened magnitudes small), and
-// re-taken exactly in double on near-ties.  Tables live in global memory
-// (L1-cached) or, when small, are staged in shared memory for the launch
-// (S and H; the bases are read only by the exact re-decision).
+// re-taken exactly in double on near-ties of the true path.  Tables live in
+// global memory (L1-cached) or, when small, are staged in shared memory for
+// the launch (S and H; the bases are read only by the exact re-decision).
 //
 // The outcome is the sequential chain itself, trial for trial:
 //   - random numbers are drawn per trial index from the TRIAL stream of
@@ -51,16 +54,35 @@
 //     pair converts exactly) and equals the sequential additions whenever
 //     ln f = 2^-k and the values stay within 53 (pair: 48) bits;
 //   - the float screen is decided only outside a margin that bounds its
-//     error.  With S within 2^-24 |S| of base - c_w, the count converted to
-//     float within 2^-24 of itself, one rounding in each fma and in the
-//     difference, and the float ln u within 2^-22 (|ln u| + 1) of ln u (u
-//     rounds with relative error below 2^-23, logf errs by at most one ulp),
-//     the screened difference errs by less than
-//         2^-21 (|c| + |n| + |S_c| + |S_n| + |ln u| + 1),
-//     half of the margin M = 2^-20 (|c| + |n| + |S_c| + |S_n| + |ln u|) +
-//     2^-20 used below.  Inside the margin the decision is re-taken from the
-//     exact difference (out of line): against the float ln u where the two
-//     are farther apart than 2^-20 (|ln u| + 1), else against ln u in double.
+//     error.  With x = S + H ln f of a bin in float, t = ln u - (x_c - x_n +
+//     v ln f), v the difference of the step's visits, errs by at most
+//       2^-24 |S| + 2^-24 (|x| + |S|) + 2^-24 |x| per bin (the screen, the
+//         count converted to float, the fma),
+//       2^-24 (|x_c| + |x_n|) (their difference),
+//       0.51 2^-20 (|ln u| + 1) (u rounds with relative error below 2^-23;
+//         __logf errs by at most 2^-21.41 in [1/2, 1] and 3 ulp below), and
+//       2^-22 |t| (the last fma and subtraction, where v ln f or t is the
+//         largest term),
+//     below 0.51 M + 2^-22 |t| with M = 2^-20 (|S_c| + |x_c| + |S_n| + |x_n| +
+//     |ln u|) + 2^-20, so the sign of t is the decision whenever |t| > M.
+//     Otherwise the decision is re-taken from the exact difference: against
+//     the float ln u where the two are farther apart than 2^-20 (|ln u| + 1),
+//     else against ln u in double.
+//
+// What bounds it: the instructions of a step (about 150 a warp at G = 32, the
+// ring's refill included) and, with few walkers, the step's dependent chain
+// (lattice -> move -> shuffles -> bin -> read -> decision -> ballots ->
+// shuffle).  Reading one bin a lane instead of two, the visit counts by three
+// comparisons, the leaf by shuffle instead of a mailbox, the trial read a step
+// ahead and near-ties looked at on the path alone took 266-302 instructions a
+// step to 150.  Sampling launches of 10^4 trials per walker, GB300, 2070 MHz,
+// before -> after: L = 8 (36 walkers, 32 lanes, staged) 0.72 -> 0.41 ms; L = 16
+// (256 walkers, 32 lanes) 0.95 -> 0.64 ms; L = 32 (2048 walkers, 32 lanes) 1.64
+// -> 1.05 ms; L = 64 (3904 walkers, 16 lanes) 2.71 -> 1.60 ms.
+// Tried and slower: the visits of recent bins in a shared-memory cache (L1
+// loses the space), prefetching the neighbourhood's lines (its instructions
+// cost what it saves), the path's end by a warp reduction, flips or stores
+// under a branch.
 #include "rewl_tab.cuh"
 
 namespace rewl {
@@ -70,42 +92,60 @@ using namespace tab;
 namespace {
 
 constexpr int RING = 128;   // trials buffered per walker
+constexpr unsigned FULL = 0xFFFFFFFFu;
+
+// The lattice in shared memory: each row is cut into nblk blocks of at most
+// 30 columns, one 32-bit word each, with the column left of the block in bit
+// 0, the block's columns from bit 1 and the column right of it after them, so
+// that a site's left neighbour, itself and its right neighbour are three
+// adjacent bits of one word whatever L is.  L = 32 needs no such copies: its
+// row is one word and the three bits are adjacent after a rotation.
+struct Blocks {
+    int n, width;   // blocks per row, columns per block (the last one may have fewer, never one)
+};
+
+__host__ __device__ __forceinline__ Blocks blocks_of(int L)
+{
+    Blocks b;
+    b.n = L <= 30 || L == 32 ? 1 : L <= 60 ? 2 : 3;
+    b.width = (L + b.n - 1) / b.n;
+    return b;
+}
+
+// Entries per row of a staged window (moves within a step change m by at most
+// 5, so rows of 16 or more keep the positions of a step apart).
+__host__ __device__ __forceinline__ int staged_ld(int wM) { return wM < 15 ? 16 : wM + 1; }
 
 // One buffered trial (16 bytes, one shared-memory vector load).  Everything
 // about a trial that does not depend on the walker's state is computed when
-// the ring is refilled.
+// the ring is refilled.  The first RING_TAIL entries are kept twice, the second
+// time behind the last one, so that a step's trials are adjacent.
+constexpr int RING_TAIL = 8;
 struct RingEntry {
-    uint32_t a;    // five 6-bit fields at bits 0, 6, 12, 18, 24:
-                   //   register lattice: bit indices i*L+j of the site and of its up,
-                   //   down, left and right neighbours;
-                   //   shared lattice: row i, column j, up row, down row, left column
-    uint32_t b;    // bits 0-5: shared lattice: right column; bits 6-25: for lag
-                   //   1..4 (5 bits each), which of (site, up, down, left, right)
-                   //   is the site of trial t - lag (one-hot, or 0)
-    uint32_t xu;   // acceptance word
+    uint32_t a;    // shared lattice: rotation that brings left, site, right to bits 0-2 | the lattice words
+                   //   of the site's row << 8, of the row above << 16 and of the row below << 24
+                   // register lattice: mask of the four neighbours, bits 0-31
+    uint32_t b;    // shared lattice: for lag 1..4 (5 bits each), which of (left, site, right, up, down) is the
+                   //   site of trial t - lag (one-hot, or 0); the site i*L+j << 20
+                   // register lattice: mask of the four neighbours, bits 32-63
+    uint32_t f;    // shared lattice, one block a row: mask of the site's bit(s) in its word
+                   // shared lattice, several blocks: the site's copy in another block: 1 | its bit << 1 |
+                   //   its word minus the site's, plus 2, << 6 (0: none)
+                   // register lattice: the site
     float lnu;     // ln u in float
 };
+static_assert(sizeof(RingEntry) == 16, "one vector load per trial");
+constexpr size_t RING_BYTES = (RING + RING_TAIL) * sizeof(RingEntry);
 
-// Per-walker exchange area of one step (shared memory, 16-byte aligned: it
-// follows the ring).  The leaf's four words are written and read as one
-// 16-byte vector.
-struct Mailbox {
-    int fsite[8];                  // register lattice: bit index flipped by trial t+k, 64 if none
-    int leafC;                     // position e << 16 | m after the last trial
-    int leafcC;                    // the path's visits of that bin
-    int leafq;                     // its H as read this step (>= 0)
-    float leafs;                   // its screen value
-};
-static_assert(offsetof(Mailbox, leafC) % 16 == 0 && (RING * sizeof(RingEntry)) % 16 == 0,
-              "the leaf's post must be 16-byte aligned");
-
-// Eq. 1 decided from the exact values (near-ties of the float screen only);
-// kept out of line so none of it runs in the common case.  ccnt and ncnt
-// are the visit counts the chain has at that point; the difference is exact
-// in double.
+// Eq. 1 decided from the exact values (near-ties of the float screen on the
+// true path only).
+// ccnt and ncnt are the visit counts the chain has at that point; the
+// difference is exact in double.  q: the trial's index (its acceptance word
+// is drawn again where ln u is needed in double).
 template <class TB>
-__device__ __noinline__ int exact_accept(const typename TB::Elem *gb, unsigned ci, int ccnt, unsigned ni, int ncnt,
-                                         double lnf, uint32_t xu, float lnu32)
+__device__ __forceinline__ int exact_accept(const typename TB::Elem *gb, unsigned ci, int ccnt, unsigned ni, int ncnt,
+                                         double lnf, float lnu32, unsigned long long q, uint32_t w, uint32_t key0,
+                                         uint32_t key1)
 {
     const double delta = fma((double)ccnt, lnf, TB::exact(gb[ci])) - fma((double)ncnt, lnf, TB::exact(gb[ni]));
     if (delta >= 0.0) return 1;
@@ -113,28 +153,22 @@ __device__ __noinline__ int exact_accept(const typename TB::Elem *gb, unsigned c
     const double band = (fabs(lu) + 1.0) * 0x1p-20;
     if (lu < delta - band) return 1;
     if (lu > delta + band) return 0;
-    return log(unit_open_d(xu)) < delta ? 1 : 0;
+    const u32x4 x = philox10((uint32_t)(q >> 1), (uint32_t)(q >> 33), w, TAG_TRIAL, key0, key1);
+    return log(unit_open_d((q & 1ull) ? x.w : x.y)) < delta ? 1 : 0;
 }
 
 template <int G>
 struct TreeShape {
-    static constexpr int DEPTH = G == 32 ? 4 : G == 16 ? 3 : G == 8 ? 2 : 1;
+    static constexpr int DEPTH = G == 32 ? 4 : G == 16 ? 3 : 2;
 };
-
-// Position code of a site for the relation codes: the bit index (register
-// lattice) or row | column << 6 (shared lattice).
-template <bool REG>
-__device__ __forceinline__ uint32_t site_code(uint32_t a)
-{
-    return REG ? (a & 63u) : (a & 0xFFFu);
-}
 
 }  // namespace
 
 // REG: the lattice (N <= 64 sites, bit i*L + j) is held in a 64-bit register
-// by every lane; otherwise it lives in shared memory, one 32-bit word per row
-// (two for L > 32).  SMT: S and H staged in shared memory for the launch.
-template <int WPR, bool SMT, int G, int PREC, bool REG>
+// by every lane; otherwise it lives in shared memory (Blocks).  SMT: S and H
+// staged in shared memory for the launch.
+// WIDE: rows of several blocks.
+template <bool SMT, int G, int PREC, bool REG, bool WIDE>
 __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, int smem_per_walker)
 {
     using TB = Tab<PREC>;
@@ -146,94 +180,164 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int gl = lane & (G - 1), grp = lane / G;
-    const unsigned gmask = GBITS << (grp * G);
     const int slot = wid * GPW + grp;   // walker slot within the block
-    const int w = blockIdx.x * ((blockDim.x >> 5) * GPW) + slot;
-    if (w >= p.nwalk || ntrials == 0) return;
-    if (!p.active[w / p.W] || p.st->done) return;
+    if (ntrials == 0 || p.st->done) return;
+    // The groups of a warp run in lockstep (every collective takes the whole
+    // warp), so a group without a walker to sample (past the last walker, or
+    // of an empty window) goes along idle: it reads a walker's data, never has
+    // a lane on the true path and writes nothing.
+    const int wany = blockIdx.x * ((blockDim.x >> 5) * GPW) + slot;
+    const int w = min(wany, p.nwalk - 1);
+    const bool idle = wany >= p.nwalk || !p.active[w / p.W];
+    if (__all_sync(FULL, idle)) return;
 
     unsigned char *base = smem_raw + (size_t)slot * smem_per_walker;
     RingEntry *ring = reinterpret_cast<RingEntry *>(base);
-    Mailbox *box = reinterpret_cast<Mailbox *>(base + RING * sizeof(RingEntry));
-    uint32_t *lat = reinterpret_cast<uint32_t *>(base + RING * sizeof(RingEntry) + sizeof(Mailbox));
-    const int L = p.L, nwords = L * WPR;
-    const int T = p.T;
+    uint32_t *lat = reinterpret_cast<uint32_t *>(base + RING_BYTES);   // nlat words and G that take the idle lanes' flips
+    const int L = p.L;
+    const Blocks bk = blocks_of(L);
+    const int nlat = REG ? 0 : L * bk.n;
     const Elem *g_base = reinterpret_cast<const Elem *>(PREC == REWL_FP64 ? (const void *)p.lng : (const void *)p.lng2)
                        + (size_t)w * p.tstride;
     int32_t *gH = p.H + (size_t)w * p.tstride;
     const float *gS = p.scr + (size_t)w * p.tstride;
-    const float *S;
-    int32_t *Hh;
-    if constexpr (SMT) {
-        float *sS = reinterpret_cast<float *>(base + RING * sizeof(RingEntry) + sizeof(Mailbox) + ((nwords * 4 + 15) & ~15));
-        int32_t *sH = reinterpret_cast<int32_t *>(sS + ((T + 3) & ~3));
-        for (int k = gl; k < T; k += G) { sS[k] = gS[k]; sH[k] = gH[k]; }
-        S = sS;
-        Hh = sH;
-    } else {
-        S = gS;
-        Hh = gH;
-    }
-    unsigned long long lat64 = 0;
-    if (REG) {
-        for (int r = 0; r < L; ++r)
-            lat64 |= (unsigned long long)p.spins[(size_t)r * p.nwalk + w] << (r * L);
-    } else {
-        for (int k = gl; k < nwords; k += G) lat[k] = p.spins[(size_t)k * p.nwalk + w];
-    }
-    __syncwarp(gmask);
-
-    const int4 R = p.rect[w / p.W];
+    // staged: (screen, visits >= 0) of each bin, rows of ld entries, with two
+    // rows before and after the window's and at least one entry after each row
+    // that are marked outside (visits -1), so a proposed bin's entry says itself
+    // whether it is in the window; a bin without a visit goes back unwritten
     const int wM = p.wM;
-    const unsigned spanE = (unsigned)(R.y - R.x), spanM = (unsigned)(R.w - R.z);
-    const unsigned Tm1 = (unsigned)(T - 1);
+    const int ld = staged_ld(wM);
+    const int nstaged = (p.wE + 4) * ld;
+    int2 *tab = reinterpret_cast<int2 *>(base + RING_BYTES + (REG ? 0 : ((nlat + G) * 4 + 15) & ~15));
+    if constexpr (SMT) {
+        #pragma unroll 4
+        for (int k = gl; k < nstaged; k += G) {
+            const int e = k / ld - 2, m = k - (e + 2) * ld;
+            const bool in = e >= 0 && e < p.wE && m < wM;
+            tab[k] = in ? make_int2(__float_as_int(gS[e * wM + m]), max(gH[e * wM + m], 0))
+                        : make_int2(0, -1);
+        }
+    }
+    // row r of the stored lattice as 64 bits
+    auto stored_row = [&](int r) -> unsigned long long {
+        unsigned long long v = p.spins[(size_t)(r * p.wpr) * p.nwalk + w];
+        if (p.wpr == 2) v |= (unsigned long long)p.spins[(size_t)(r * 2 + 1) * p.nwalk + w] << 32;
+        return v;
+    };
+    uint32_t lo = 0, hi = 0;            // REG: the committed lattice
+    if (REG) {
+        unsigned long long v = 0;
+        for (int r = 0; r < L; ++r) v |= stored_row(r) << (r * L);
+        lo = (uint32_t)v;
+        hi = (uint32_t)(v >> 32);
+    } else {
+        for (int k = gl; k < nlat; k += G) {
+            const int r = k / bk.n, q = k - r * bk.n, c0 = q * bk.width;
+            const unsigned long long v = stored_row(r);
+            if (L == 32) {
+                lat[k] = (uint32_t)v;
+            } else {
+                unsigned long long x = c0 ? v >> (c0 - 1) : (v << 1) | ((v >> (L - 1)) & 1ull);
+                if (L - c0 <= bk.width) x |= (v & 1ull) << (L - c0 + 1);
+                lat[k] = (uint32_t)x;
+            }
+        }
+    }
+    __syncwarp();
+
+    // positions: staged, the bin's entry; else (e - e0) << 16 | (m - m0).  A
+    // move changes e by de and m by dm, the position by de * erow + dm.
+    const int4 R = p.rect[w / p.W];
+    const int erow = SMT ? ld : 65536;
+    const int estep = wM - 65536;       // global tables: index = position + e * estep
+    const unsigned Tm1 = (unsigned)(p.T - 1);
     const double lnf = p.st->lnf;
     const float lnf32 = __double2float_rn(lnf);
     const uint32_t N = (uint32_t)p.N;
     const uint32_t divL = p.divL;
 
-    // this lane's node of the tree and the lanes holding its history's trials
+    // This lane's node of the tree.  Lane G-1 holds none: it never accepts and
+    // its move is 0.
     const int dl = 31 - __clz(gl + 1);
-    const int hist = gl + 1 - (1 << dl);
-    int srck[DEPTH];
+    const bool node = gl < G - 1;
+    const int hist = node ? gl + 1 - (1 << dl) : 0;
+    const int spanp = node ? ((R.y - R.x) << 16) | (R.w - R.z) : (int)0xC0000000;
+    // Lanes of the accepted trials of the history, the latest first (lane G-1
+    // where there are fewer), and how many of the step's trials end in the
+    // bins the history passes: n0 in the current one since the last accepted
+    // trial, n1, n2, n3 in the ones before it.
+    int src[DEPTH], seg[DEPTH + 1];
     #pragma unroll
-    for (int k = 0; k < DEPTH; ++k) srck[k] = grp * G + (1 << k) - 1 + (hist & ((1 << k) - 1));
-    // the lane is on the true path iff the ballot bits of its ancestors
-    // (lane 2^k - 1 + (h mod 2^k) at depth k < d) are the outcomes its
-    // history assumes: anc marks the ancestors, want holds those outcomes
+    for (int j = 0; j < DEPTH; ++j) src[j] = grp * G + G - 1;
+    #pragma unroll
+    for (int j = 0; j <= DEPTH; ++j) seg[j] = 0;
+    {
+        int j = 0, last = dl;            // last: the trial after the segment's end
+        for (int k = DEPTH - 1; k >= 0; --k)
+            if (node && k < dl && ((hist >> k) & 1)) {
+                #pragma unroll
+                for (int q = 0; q < DEPTH; ++q)
+                    if (q == j) { src[q] = grp * G + (1 << k) - 1 + (hist & ((1 << k) - 1)); seg[q] = last - k; }
+                last = k;
+                ++j;
+            }
+        #pragma unroll
+        for (int q = 0; q <= DEPTH; ++q)
+            if (node && q == j) seg[q] = last;
+    }
+    const int n0 = seg[0], n1 = seg[1], n2 = DEPTH >= 3 ? seg[2] : 0, n3 = DEPTH >= 4 ? seg[DEPTH >= 4 ? 3 : 0] : 0;
+    // On the true path iff the ballot bits of the ancestors (lane 2^k - 1 +
+    // (h mod 2^k) at depth k < d) are the outcomes the history assumes: anc
+    // marks the ancestors, want holds those outcomes.  Lane G-1 of the group
+    // never accepts: asking for its acceptance takes a lane off every path.
+    const unsigned never = 1u << (grp * G + G - 1);
     unsigned anc = 0, want = 0;
     #pragma unroll
     for (int k = 0; k <= DEPTH; ++k)
         if (k < dl) {
-            const int a = (1 << k) - 1 + (hist & ((1 << k) - 1));
+            const int a = grp * G + (1 << k) - 1 + (hist & ((1 << k) - 1));
             anc |= 1u << a;
             want |= (unsigned)((hist >> k) & 1) << a;
         }
-    // relation fields of the lags whose trials the history accepts: trial
-    // t+k (k < d) is lag d - k of this lane's trial
-    uint32_t sel = 0;
+    if (idle || !node) { anc |= never; want |= never; }
+    // A lane that accepts on the path writes the visits of the bin it enters,
+    // lane G-1 those of the step's first bin.  later: the trials after the
+    // lane's; rank: order among the bins of the path that could be the same one
+    // (those an even number of accepted trials apart, and visited in the step).
+    const bool first = !node && !idle;
+    const int later = node ? dl + 1 : 0;
+    const int rank = node ? (__popc(hist) + 1 - (dl == 0 ? 1 : hist & 1)) >> 1 : 0;
+    const int hacc = node ? hist | (1 << dl) : 0;
+    // relation fields of the lags whose trials the history accepts: trial t+k
+    // (k < d) is lag d - k of this lane's trial; REG: the accepted trials
+    uint32_t sel = 0, flip[DEPTH];
     #pragma unroll
-    for (int k = 0; k <= DEPTH; ++k)
-        if (k < dl && ((hist >> k) & 1)) sel |= 0x1Fu << (5 * (dl - k - 1));
+    for (int k = 0; k < DEPTH; ++k) {
+        const bool on = node && k < dl && ((hist >> k) & 1);
+        if (on) sel |= 0x1Fu << (5 * (dl - k - 1));
+        flip[k] = on ? FULL : 0u;
+    }
+    // move (position difference) of a trial whose five spins (left, site,
+    // right, up, down) are the lane's number: looked up by shuffle
+    const int nup_l = __popc(lane & 0x1D);
+    const int lut = (lane & 2) ? (nup_l - 2) * erow - 1 : (2 - nup_l) * erow + 1;
+    const int mvA = node ? erow : 0, mvB = node ? 2 * erow + 1 : 0;   // REG: the move is +-(nup mvA - mvB)
 
-    // committed state (uniform over the group); positions are e << 16 | m
-    int P0 = (p.we[w] << 16) | p.wm[w];
-    int ci = ((P0 >> 16) - R.x) * wM + ((P0 & 0xFFFF) - R.z);
-    int lq = max(Hh[ci], 0);        // H of the current bin, visits of this step excluded
-    int hq = 0;                     // visits of the current bin not yet written to H
-    float base32 = S[ci];
+    // committed position (uniform over the group)
+    int P0 = (p.we[w] - R.x + (SMT ? 2 : 0)) * erow + (p.wm[w] - R.z);
     const unsigned long long t0 = p.wt[w];
     const unsigned r0 = (unsigned)t0 & RMASK;
-    unsigned u = 0;                 // trials done in this launch
-    unsigned ufill = 0;             // ring holds trials [t0 - (t0 & 1), t0 + ufill)
     const unsigned long long c0 = t0 >> 1;   // first Philox call
-    unsigned cfill = 0;             // calls done
-    int err = 0;
+    unsigned u = 0;                 // trials done in this launch
+    unsigned cfill = 0;             // calls done: the ring holds trials t0 - (t0 & 1) + [0, 2 cfill)
+    unsigned end = 1u << (DEPTH + 1);
+    int err = 0;                    // sign: a count passed INT_MAX
 
     while (u < ntrials) {
-        // ---- refill the ring: 32 Philox calls = 64 trials
-        if (ufill < u + 32) {
-            #pragma unroll
+        // ---- refill the ring: 32 Philox calls = 64 trials (the test leaves
+        // the parity of t0 out, so the warp's groups refill together)
+        if (2 * cfill < u + 33) {
+            #pragma unroll 1
             for (int r = 0; r < 32 / G; ++r) {
                 const unsigned long long c = c0 + cfill + (unsigned)(gl + r * G);
                 const u32x4 x = philox10((uint32_t)c, (uint32_t)(c >> 32), (uint32_t)w, TAG_TRIAL, p.key0, p.key1);
@@ -244,222 +348,284 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
                     const uint32_t i = __umulhi(site, divL);
                     const uint32_t j = site - i * (uint32_t)L;
                     const uint32_t iu = i == 0 ? L - 1 : i - 1, id = i == (uint32_t)L - 1 ? 0 : i + 1;
-                    const uint32_t jl = j == 0 ? L - 1 : j - 1, jr = j == (uint32_t)L - 1 ? 0 : j + 1;
                     RingEntry en;
                     if (REG) {
-                        en.a = site | ((iu * L + j) << 6) | ((id * L + j) << 12) | ((i * L + jl) << 18) | ((i * L + jr) << 24);
-                        en.b = 0;
+                        const uint32_t jl = j == 0 ? L - 1 : j - 1, jr = j == (uint32_t)L - 1 ? 0 : j + 1;
+                        const unsigned long long nb = (1ull << (iu * L + j)) | (1ull << (id * L + j))
+                                                    | (1ull << (i * L + jl)) | (1ull << (i * L + jr));
+                        en.a = (uint32_t)nb;
+                        en.b = (uint32_t)(nb >> 32);
+                        en.f = site;
                     } else {
-                        en.a = i | (j << 6) | (iu << 12) | (id << 18) | (jl << 24);
-                        en.b = jr;
+                        en.b = site << 20;
+                        if (WIDE) {
+                            // the first column of a block is also the bit after the previous block's last
+                            // column, the last one also bit 0 of the next block
+                            const uint32_t q = (uint32_t)((int)j >= bk.width) + (uint32_t)((int)j >= 2 * bk.width);
+                            const uint32_t amt = j - q * bk.width, qn = (uint32_t)bk.n - 1u;
+                            en.a = amt | ((i * bk.n + q) << 8) | ((iu * bk.n + q) << 16) | ((id * bk.n + q) << 24);
+                            const bool fc = amt == 0, lc = (int)amt == bk.width - 1 || (int)j == L - 1;
+                            const uint32_t qo = fc ? (q == 0 ? qn : q - 1) : (q == qn ? 0u : q + 1);
+                            const uint32_t bit = fc ? (q == 0 ? (uint32_t)L - qn * bk.width : (uint32_t)bk.width) + 1u : 0u;
+                            en.f = fc || lc ? 1u | (bit << 1) | ((qo + 2u - q) << 6) : 0u;
+                        } else {
+                            const uint32_t amt = L == 32 ? (j + 31u) & 31u : j;
+                            en.a = amt | (i << 8) | (iu << 16) | (id << 24);
+                            en.f = __funnelshift_l(2u, 2u, amt);
+                            if (L != 32) en.f |= (j == 0 ? 2u << L : 0u) | (uint32_t)(j == (uint32_t)L - 1);
+                        }
                     }
-                    en.xu = xu;
-                    en.lnu = logf(__fmaf_rn(__uint2float_rn(xu), 0x1p-32f, 0x1p-33f));
-                    ring[(unsigned)(2 * c + hh) & RMASK] = en;
+                    en.lnu = __logf(__fmaf_rn(__uint2float_rn(xu), 0x1p-32f, 0x1p-33f));
+                    const unsigned at = (unsigned)(2 * c + hh) & RMASK;
+                    ring[at] = en;
+                    if (at < RING_TAIL) ring[at + RING] = en;
                 }
             }
-            __syncwarp(gmask);
-            // relation codes of the 64 new trials to the DEPTH trials before each
-            #pragma unroll
-            for (int r = 0; r < 64 / G; ++r) {
-                const unsigned q = (unsigned)(2 * (c0 + cfill)) + (unsigned)(gl + r * G);
-                const uint32_t a = ring[q & RMASK].a, b = ring[q & RMASK].b;
-                uint32_t pos[5];
-                if (REG) {
+            __syncwarp();
+            if (!REG) {
+                // relation codes of the 64 new trials to the DEPTH trials before each
+                #pragma unroll 1
+                for (int r = 0; r < 64 / G; ++r) {
+                    const unsigned q = (unsigned)(2 * (c0 + cfill)) + (unsigned)(gl + r * G);
+                    const unsigned at = q & RMASK;
+                    const uint32_t b = ring[at].b, site = b >> 20;
+                    const uint32_t i = __umulhi(site, divL);
+                    const uint32_t j = site - i * (uint32_t)L;
+                    const uint32_t pos[5] = {j == 0 ? site + L - 1 : site - 1, site, j == (uint32_t)L - 1 ? site + 1 - L : site + 1,
+                                             i == 0 ? site + N - L : site - L, i == (uint32_t)L - 1 ? site + L - N : site + L};
+                    uint32_t rel = 0;
                     #pragma unroll
-                    for (int f = 0; f < 5; ++f) pos[f] = (a >> (6 * f)) & 63u;
-                } else {
-                    const uint32_t row = a & 63u, colbits = a & (63u << 6);
-                    pos[0] = a & 0xFFFu;
-                    pos[1] = ((a >> 12) & 63u) | colbits;
-                    pos[2] = ((a >> 18) & 63u) | colbits;
-                    pos[3] = row | (((a >> 24) & 63u) << 6);
-                    pos[4] = row | ((b & 63u) << 6);
+                    for (int lag = 1; lag <= DEPTH; ++lag) {
+                        const uint32_t f = ring[(q - lag) & RMASK].b >> 20;
+                        #pragma unroll
+                        for (int k = 0; k < 5; ++k)
+                            if (f == pos[k]) rel |= 1u << (5 * (lag - 1) + k);
+                    }
+                    rel |= site << 20;
+                    ring[at].b = rel;
+                    if (at < RING_TAIL) ring[at + RING].b = rel;
                 }
-                uint32_t rel = 0;
-                #pragma unroll
-                for (int lag = 1; lag <= DEPTH; ++lag) {
-                    const uint32_t f = site_code<REG>(ring[(q - lag) & RMASK].a);
-                    uint32_t oh = 0;
-                    #pragma unroll
-                    for (int k = 0; k < 5; ++k) oh |= (uint32_t)(f == pos[k]) << k;
-                    rel |= oh << (5 * (lag - 1));
-                }
-                ring[q & RMASK].b = b | (rel << 6);
             }
             cfill += 32;
-            ufill = 2 * cfill - (unsigned)(t0 & 1ull);
-            __syncwarp(gmask);
+            __syncwarp();
         }
-        const unsigned left = ntrials - u;
-        const int D = left > (unsigned)DEPTH ? DEPTH : (int)left - 1;
-        const unsigned rb = r0 + u;
-
-        // ---- 1. own trial under own history: the five spins
-        const RingEntry me = ring[(rb + dl) & RMASK];
-        uint32_t v5;
-        if (REG) {
-            v5 = ((uint32_t)(lat64 >> (me.a & 63u)) & 1u)
-               | (((uint32_t)(lat64 >> ((me.a >> 6) & 63u)) & 1u) << 1)
-               | (((uint32_t)(lat64 >> ((me.a >> 12) & 63u)) & 1u) << 2)
-               | (((uint32_t)(lat64 >> ((me.a >> 18) & 63u)) & 1u) << 3)
-               | (((uint32_t)(lat64 >> ((me.a >> 24) & 63u)) & 1u) << 4);
+        // steps until the ring runs low or the launch ends; its last step may
+        // be a short one, whose lanes past the last trial leave the path
+        unsigned nsteps = (2 * cfill - 1 - u) / (DEPTH + 1);
+        if (ntrials - u <= (unsigned)DEPTH) {
+            nsteps = 1;
+            end = 1u << (ntrials - u);
+            if (dl >= (int)(ntrials - u)) { anc |= never; want |= never; }
         } else {
-            const uint32_t i = me.a & 63u, j = (me.a >> 6) & 63u, iu = (me.a >> 12) & 63u, id = (me.a >> 18) & 63u;
-            const uint32_t jl = (me.a >> 24) & 63u, jr = me.b & 63u;
-            const uint32_t qj = (WPR == 1) ? 0 : (j >> 5);
-            const uint32_t wc = lat[i * WPR + qj], wu = lat[iu * WPR + qj], wd = lat[id * WPR + qj];
-            const uint32_t wl = (WPR == 1) ? wc : lat[i * WPR + (jl >> 5)];
-            const uint32_t wr = (WPR == 1) ? wc : lat[i * WPR + (jr >> 5)];
-            v5 = ((wc >> (j & 31)) & 1u) | (((wu >> (j & 31)) & 1u) << 1) | (((wd >> (j & 31)) & 1u) << 2)
-               | (((wl >> (jl & 31)) & 1u) << 3) | (((wr >> (jr & 31)) & 1u) << 4);
+            nsteps = min(nsteps, (ntrials - u) / (DEPTH + 1));
         }
-        {
-            const uint32_t corr = (me.b >> 6) & sel;
-            v5 ^= (corr ^ (corr >> 5) ^ (corr >> 10) ^ (corr >> 15)) & 0x1Fu;
-        }
-        const int sup = (int)(v5 & 1u);
-        const int nup = __popc(v5 & 0x1Eu);
-        const int de_own = sup ? nup - 2 : 2 - nup;
-        const int dm_own = sup ? -1 : 1;
-        const int pk = de_own * 65536 + dm_own;   // move as a position difference
-
-        // ---- 2. the history's earlier trials: the move of trial k under the
-        // history's first k outcomes is the own move of lane 2^k - 1 + (h mod 2^k);
-        // a history that accepts a move out of the window is never the true path
-        int Pc = P0;
-        int vb[DEPTH];               // position after each earlier trial (-1 past the own depth)
-        #pragma unroll
-        for (int k = 0; k < DEPTH; ++k) {
-            const int x = __shfl_sync(gmask, pk, srck[k]);
-            if ((hist >> k) & 1) Pc += x;
-            vb[k] = k < dl ? Pc : -1;
-        }
-        const int Pn = Pc + pk;
-        const int ce = Pc >> 16, cm = Pc & 0xFFFF;
-        const int cidx = (ce - R.x) * wM + (cm - R.z);
-        const int nidx = cidx + de_own * wM + dm_own;
-        const bool live = dl <= D && (unsigned)(ce + de_own - R.x) <= spanE && (unsigned)(cm + dm_own - R.z) <= spanM;
-
-        // ---- 3. decision of the own trial (Eq. 1); off-path lanes may hold
-        // positions outside the window, so their reads are clamped
-        const unsigned cu = min((unsigned)cidx, Tm1), nu = min((unsigned)nidx, Tm1);
-        // a lane whose bin is the walker's committed bin takes S and H from
-        // registers (base32, lq); with the tables in global memory it also
-        // skips their load (in shared memory the predicate costs more than the load)
-        const bool c0p = !SMT && Pc == P0, n0p = !SMT && Pn == P0;
-        const float cs_m = c0p ? 0.f : S[cu], ns_m = n0p ? 0.f : S[nu];
-        const int hc = c0p ? 0 : max(Hh[cu], 0), hn = n0p ? 0 : max(Hh[nu], 0);
-        int vcur = 0, vnew = 0;
-        #pragma unroll
-        for (int k = 0; k < DEPTH; ++k) {
-            vcur += (vb[k] == Pc);
-            vnew += (vb[k] == Pn);
-        }
-        const bool c0b = Pc == P0, n0b = Pn == P0;
-        const float cs = c0b ? base32 : cs_m, ns = n0b ? base32 : ns_m;
-        const int ccnt = vcur + (c0b ? lq : hc), ncnt = vnew + (n0b ? lq : hn);
-        const float c32 = __fmaf_rn(__int2float_rn(ccnt), lnf32, cs);
-        const float n32 = __fmaf_rn(__int2float_rn(ncnt), lnf32, ns);
-        const float d32 = __fsub_rn(c32, n32);
-        // the terms known before c and n are summed first (shorter chain; the
-        // margin's factor-two slack over the error bound covers either order)
-        const float M = __fmaf_rn((fabsf(c32) + fabsf(n32)) + (fabsf(cs) + fabsf(ns) + fabsf(me.lnu)), 0x1p-20f,
-                                  0x1p-20f);
-        int acc = (me.lnu < d32 - M) ? 1 : 0;
-        if (live && !acc && !(me.lnu > d32 + M))
-            acc = exact_accept<TB>(g_base, cu, ccnt, nu, ncnt, lnf, me.xu, me.lnu);
-        acc = live ? acc : 0;
-        const int after = acc ? Pn : Pc;          // position after the own trial, under the own history
-
-        // ---- the true path: the lanes whose ancestors decided as their history assumes
-        const unsigned bal = (__ballot_sync(gmask, acc) >> (grp * G)) & GBITS;
-        const bool onp = dl <= D && ((bal ^ want) & anc) == 0u;
-
-        // ---- commit: the on-path lane of depth k takes trial t+k.  Its bin has
-        // cupto path visits up to and including this trial, so its H becomes
-        // cupto plus the H it had (the current bin: lq).
-        const int aq = acc ? hn : hc;             // H of `after` as read (unless it is the current bin)
-        const int cupto = (acc ? vnew : vcur) + 1;
-        const int val = cupto + (after == P0 ? lq : aq);
-        const unsigned aidx = acc ? nu : cu;
-        if (onp) {
-            if (REG) box->fsite[dl] = acc ? (int)(me.a & 63u) : 64;
-            if (dl == D)      // one 16-byte store: position, visits, H, screen
-                *reinterpret_cast<int4 *>(&box->leafC) = make_int4(after, cupto, aq, __float_as_int(acc ? ns : cs));
-            err |= val < 0;
-        }
-        // H of the bins visited in this step, in path order: the pending count of
-        // the start bin, then each trial's bin with its visits so far; a bin
-        // visited again later in the step is overwritten with the larger count,
-        // so every bin ends with all its visits (the warp barriers order the
-        // stores of different lanes to one address)
-        if (gl == 0 && hq > 0) Hh[ci] = lq;
-        #pragma unroll
-        for (int k = 0; k <= DEPTH; ++k) {
-            __syncwarp(gmask);
-            if (onp && dl == k) Hh[aidx] = val;
-        }
-        __syncwarp(gmask);
-        const int4 lb = *reinterpret_cast<const int4 *>(&box->leafC);   // the leaf's post
-        const int C = lb.x, cC = lb.y;
-        if (REG) {
-            #pragma unroll
-            for (int k = 0; k <= DEPTH; ++k) {
-                if (k <= D) {
-                    const int f = box->fsite[k];
-                    lat64 ^= (unsigned long long)(f < 64) << (f & 63);
+        // what the step's trials need that does not depend on the state is read
+        // a step ahead: the lane's trial and, REG, the sites its history flips
+        RingEntry nxt;
+        uint32_t nlo = 0, nhi = 0;
+        auto ahead = [&](unsigned at) {
+            const RingEntry *now = ring + (at & RMASK);
+            nxt = now[dl];
+            if (REG) {
+                nlo = nhi = 0;
+                #pragma unroll
+                for (int k = 0; k < DEPTH; ++k) {
+                    const unsigned long long b = 1ull << now[k].f;
+                    nlo ^= (uint32_t)b & flip[k];
+                    nhi ^= (uint32_t)(b >> 32) & flip[k];
                 }
             }
-        } else if (onp && acc) {
-            const uint32_t fi = me.a & 63u, fj = (me.a >> 6) & 63u;
-            atomicXor(&lat[fi * WPR + ((WPR == 1) ? 0 : (fj >> 5))], 1u << (fj & 31));
+        };
+        ahead(r0 + u);
+        #pragma unroll 2
+        for (unsigned it = 0; it < nsteps; ++it) {
+        // ---- 1. own trial under own history: its move, as a position difference
+        const RingEntry me = nxt;
+        uint32_t hlo = 0, hhi = 0, olo = 0, ohi = 0;   // REG: the lattice under the history; the site's bit
+        int pk;
+        if (REG) {
+            hlo = lo ^ nlo;
+            hhi = hi ^ nhi;
+            const unsigned long long o = 1ull << me.f;
+            olo = (uint32_t)o;
+            ohi = (uint32_t)(o >> 32);
+            const bool sup = ((hlo & olo) | (hhi & ohi)) != 0u;
+            pk = (__popc(hlo & me.a) + __popc(hhi & me.b)) * (sup ? mvA : -mvA) + (sup ? -mvB : mvB);
+        } else {
+            const uint32_t wc = lat[(me.a >> 8) & 0xFFu], wu = lat[(me.a >> 16) & 0xFFu], wd = lat[me.a >> 24];
+            uint32_t v5 = (__funnelshift_r(wc, wc, me.a) & 7u) | (__funnelshift_r(wu, wu, me.a - 2u) & 8u)
+                        | (__funnelshift_r(wd, wd, me.a - 3u) & 16u);
+            uint32_t corr = me.b & sel;
+            if (DEPTH > 2) corr ^= corr >> 10;
+            corr ^= corr >> 5;
+            v5 ^= corr;
+            pk = __shfl_sync(FULL, lut, v5);        // (the low five bits select)
+            if (!node) pk = 0;
         }
-        // the group adopts the state after the last trial
-        {
-            const bool same = C == P0;
-            const int nlq = (same ? lq : lb.z) + cC;
-            const float ns32 = __int_as_float(lb.w);
-            hq = same ? hq + cC : cC;
-            lq = nlq;
-            err |= nlq < 0;
-            if (!same) {
-                base32 = ns32;
-                ci = ((C >> 16) - R.x) * wM + ((C & 0xFFFF) - R.z);
+
+        // ---- 2. position under the history (Pc) and after the own move (Pn),
+        // and by how much the step's earlier trials visited the current bin more
+        // often than the proposed one (the bin before the last 2 accepted trials
+        // is the current one again iff their moves cancel, and so on)
+        int y[DEPTH];
+        #pragma unroll
+        for (int j = 0; j < DEPTH; ++j) y[j] = __shfl_sync(FULL, pk, src[j]);
+        const int z2 = y[0] + y[1];
+        const int zl = DEPTH >= 4 ? y[DEPTH >= 3 ? 2 : 0] + y[DEPTH >= 4 ? 3 : 0] : DEPTH >= 3 ? y[DEPTH >= 3 ? 2 : 0] : 0;
+        const int Pc = P0 + z2 + zl, Pn = (P0 + pk) + z2 + zl;
+        int vnew = pk + y[0] == 0 ? n1 : 0;
+        if (DEPTH >= 4) vnew += pk + z2 + y[DEPTH >= 3 ? 2 : 0] == 0 ? n3 : 0;
+        int vcur = n0;
+        if (DEPTH >= 3) vcur += z2 == 0 ? n2 : 0;
+
+        // ---- 3. decision of the own trial (Eq. 1).  Off-path lanes may hold
+        // positions outside the window: clamped reads.  With global tables a lane
+        // reads the proposed bin alone: the current one is the bin the history's
+        // last accepted trial proposed, or the step's first bin, which lane G-1
+        // reads; with staged ones a second read is cheaper than that shuffle.
+        unsigned nu;
+        bool live = node;                 // the proposed bin is in the window
+        float xn, mn, xc, mc;
+        int hn;
+        if constexpr (SMT) {
+            nu = min((unsigned)Pn, (unsigned)nstaged - 1u);
+            const int2 n = tab[nu], c = tab[min((unsigned)Pc, (unsigned)nstaged - 1u)];
+            hn = n.y;
+            live = node && n.y >= 0;
+            xn = __fmaf_rn(__int2float_rn(n.y), lnf32, __int_as_float(n.x));
+            xc = __fmaf_rn(__int2float_rn(c.y), lnf32, __int_as_float(c.x));
+            mn = fabsf(__int_as_float(n.x)) + fabsf(xn);
+            mc = fabsf(__int_as_float(c.x)) + fabsf(xc);
+        } else {
+            nu = min((unsigned)(Pn + (Pn >> 16) * estep), Tm1);
+            const float sn = gS[nu];
+            hn = max(gH[nu], 0);
+            live = ((Pn | (spanp - Pn)) & 0x80008000) == 0;
+            xn = __fmaf_rn(__int2float_rn(hn), lnf32, sn);
+            mn = fabsf(sn) + fabsf(xn);
+            xc = __shfl_sync(FULL, xn, src[0]);
+            mc = __shfl_sync(FULL, mn, src[0]);
+        }
+        ahead(r0 + u + DEPTH + 1);
+        const float t32 = __fsub_rn(me.lnu, __fmaf_rn(__int2float_rn(vcur - vnew), lnf32, __fsub_rn(xc, xn)));
+        const float M = __fmaf_rn(mc + mn + fabsf(me.lnu), 0x1p-20f, 0x1p-20f);
+        bool acc = live && t32 < 0.0f;
+        bool near = live && !(fabsf(t32) > M);      // (not a number counts as near)
+
+        // ---- the true path: the lanes whose ancestors decided as their
+        // histories assume, and the state after its last trial
+        unsigned bal, nearb, pm, path;
+        bool onp;
+        int Pa;
+        uint32_t lo2 = 0, hi2 = 0;
+        auto follow = [&]() {
+            bal = __ballot_sync(FULL, acc);
+            nearb = __ballot_sync(FULL, near);
+            onp = ((bal ^ want) & anc) == 0u;
+            pm = __ballot_sync(FULL, onp);
+            const int leaf = 31 - __clz(pm & (GBITS << (grp * G)));
+            Pa = __shfl_sync(FULL, acc ? Pn : Pc, leaf);
+            if (REG) {
+                lo2 = __shfl_sync(FULL, acc ? hlo ^ olo : hlo, leaf);
+                hi2 = __shfl_sync(FULL, acc ? hhi ^ ohi : hhi, leaf);
             }
-            P0 = C;
+            path = __shfl_sync(FULL, acc ? hacc : hist, leaf);   // bit k: trial k accepted
+        };
+        follow();
+        while (pm & nearb) {              // near-ties on the path are decided exactly
+            if (onp && near) {
+                unsigned ib, jb;          // the bins' entries in the window's table
+                int hc;
+                if constexpr (SMT) {
+                    ib = (unsigned)(Pc - (Pc / ld) * (ld - wM) - 2 * wM);
+                    jb = (unsigned)(Pn - (Pn / ld) * (ld - wM) - 2 * wM);
+                    hc = tab[Pc].y;
+                } else {
+                    ib = (unsigned)(Pc + (Pc >> 16) * estep);
+                    jb = nu;
+                    hc = max(gH[ib], 0);
+                }
+                acc = exact_accept<TB>(g_base, ib, hc + vcur, jb, hn + vnew, lnf, me.lnu, t0 + u + dl, (uint32_t)w, p.key0,
+                                       p.key1);
+                near = false;
+            }
+            __syncwarp();
+            follow();
         }
-        __syncwarp(gmask);
-        u += (unsigned)(D + 1);
+
+        // ---- commit: the visits of the path's bins are written: the count a bin
+        // had, plus its earlier visits in the step, plus those until the path
+        // leaves it.  A bin the path comes back to is written again with the
+        // larger count; the stores of such bins are ordered by rank.
+        P0 = Pa;
+        if (REG) {
+            lo = lo2;
+            hi = hi2;
+        } else {
+            // lanes without a flip go to a word of their own (a branch would
+            // cost the warp more than the added traffic)
+            const bool flip = onp && acc;
+            uint32_t *const own = lat + nlat + gl, *const word = lat + ((me.a >> 8) & 0xFFu);
+            atomicXor(flip ? word : own, WIDE ? 2u << (me.a & 31u) : me.f);
+            if (WIDE) atomicXor(flip && (me.f & 1u) ? word + (int)(me.f >> 6) - 2 : own, 1u << ((me.f >> 1) & 31u));
+        }
+        const int stay = __ffs((path | end) >> later) - (node ? 0 : 1);
+        const bool st = node ? onp && acc : first && stay > 0;
+        const int val = hn + vnew + stay;
+        if (st) err |= val;
+        #pragma unroll
+        for (int k = 0; k < (DEPTH >= 4 ? 3 : 2); ++k) {
+            if (k) __syncwarp();
+            if (st && rank == k) {
+                if constexpr (SMT) tab[nu].y = val;
+                else gH[nu] = val;
+            }
+        }
+        __syncwarp();
+        u += (unsigned)(DEPTH + 1);
+        }
     }
 
-    // ---- flush the current bin and the state
-    if (gl == 0 && hq > 0) Hh[ci] = lq;
-    __syncwarp(gmask);
+    // ---- the state
+    if (__any_sync(FULL, err < 0) && lane == 0) atomicOr(&p.st->error, ERR_OVERFLOW);
+    __syncwarp();
+    if (idle) return;
     if constexpr (SMT) {
-        for (int k = gl; k < T; k += G) gH[k] = Hh[k];
+        for (int k = gl + 2 * ld; k < nstaged - 2 * ld; k += G) {
+            const int e = k / ld - 2, m = k - (e + 2) * ld, h = tab[k].y;
+            if (m < wM && h > 0) gH[e * wM + m] = h;
+        }
     }
-    if (REG) {
-        for (int r = gl; r < L; r += G)
-            p.spins[(size_t)r * p.nwalk + w] = (uint32_t)(lat64 >> (r * L)) & (uint32_t)((1ull << L) - 1);
-    } else {
-        for (int k = gl; k < nwords; k += G) p.spins[(size_t)k * p.nwalk + w] = lat[k];
+    for (int r = gl; r < L; r += G) {
+        unsigned long long v;
+        if (REG) {
+            v = ((((unsigned long long)hi << 32) | lo) >> (r * L)) & ((1ull << L) - 1);
+        } else if (L == 32) {
+            v = lat[r];
+        } else {
+            v = 0;
+            for (int q = 0; q < bk.n; ++q)
+                v |= (unsigned long long)((lat[r * bk.n + q] >> 1) & ((1u << bk.width) - 1u)) << (q * bk.width);
+            if (L < 64) v &= (1ull << L) - 1;
+        }
+        p.spins[(size_t)(r * p.wpr) * p.nwalk + w] = (uint32_t)v;
+        if (p.wpr == 2) p.spins[(size_t)(r * 2 + 1) * p.nwalk + w] = (uint32_t)(v >> 32);
     }
     if (gl == 0) {
-        p.we[w] = P0 >> 16;
-        p.wm[w] = P0 & 0xFFFF;
-        p.wt[w] = t0 + u;
+        const int e = P0 / erow;
+        p.we[w] = e - (SMT ? 2 : 0) + R.x;
+        p.wm[w] = P0 - e * erow + R.z;
+        p.wt[w] = t0 + ntrials;
     }
-    err = __any_sync(gmask, err);
-    if (gl == 0 && err) atomicOr(&p.st->error, ERR_OVERFLOW);
 }
 
-// Shared memory per walker: ring, mailbox, lattice (16-byte padded) and, when
-// staged, S (4 bytes per bin, padded to 16 bytes) and H (4 bytes per bin).
-size_t tree_smem_per_warp(const Params &p, bool smt)
+// Shared memory per walker: ring, lattice (16-byte padded) and, when staged,
+// S and H (8 bytes per entry).
+size_t tree_smem_per_warp(const Params &p, bool smt, int group)
 {
-    size_t b = RING * sizeof(RingEntry) + sizeof(Mailbox) + (((size_t)p.nwords * 4 + 15) & ~(size_t)15);
-    if (smt) b += (((size_t)p.T + 3) & ~(size_t)3) * 4 + (size_t)p.T * 4;
+    const size_t nlat = p.lattice_reg ? 0 : (size_t)p.L * blocks_of(p.L).n + group;
+    size_t b = RING_BYTES + ((nlat * 4 + 15) & ~(size_t)15);
+    if (smt) b += (size_t)(p.wE + 4) * staged_ld(p.wM) * 8;
     return (b + 15) & ~(size_t)15;
 }
 
@@ -470,11 +636,16 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
 {
     if (p.precision != REWL_FP64 && p.precision != REWL_F32X2) return cudaErrorInvalidValue;
     if (group != 8 && group != 16 && group != 32) group = 32;
-    const size_t per = tree_smem_per_warp(p, smt);
     const int gpw = 32 / group;
+    const size_t max_smem = 227 * 1024;
+    // a window whose bins fit in a block's shared memory, but not with the
+    // entries around them, is sampled from global memory
+    if (smt && tree_smem_per_warp(p, true, group) * gpw > max_smem
+        && (RING * sizeof(RingEntry) + 48 + (((size_t)p.nwords * 4 + 15) & ~(size_t)15) + 8 * (size_t)p.T) * gpw <= max_smem)
+        smt = false;
+    const size_t per = tree_smem_per_warp(p, smt, group);
     if (warps <= 0) warps = smt ? 1 : 4;
     // no more warps per block than the shared memory of one block holds
-    const size_t max_smem = 227 * 1024;
     while (warps > 1 && per * (size_t)gpw * warps > max_smem) --warps;
     if (per * (size_t)gpw * warps > max_smem) return cudaErrorInvalidValue;
     const size_t smem = per * (size_t)gpw * warps;
@@ -489,24 +660,22 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
         kern<<<blocks, threads, smem, s>>>(p, (unsigned)ntrials, (int)per);
         return cudaGetLastError();
     };
-#define REWL_TREE_G(W_, S_, P_)                                            \
-    if (p.lattice_reg && W_ == 1) {                                        \
-        if (group == 32) return go(k_sweep_tree<1, S_, 32, P_, true>);     \
-        if (group == 16) return go(k_sweep_tree<1, S_, 16, P_, true>);     \
-        return go(k_sweep_tree<1, S_, 8, P_, true>);                       \
-    }                                                                      \
-    if (group == 32) return go(k_sweep_tree<W_, S_, 32, P_, false>);       \
-    if (group == 16) return go(k_sweep_tree<W_, S_, 16, P_, false>);       \
-    return go(k_sweep_tree<W_, S_, 8, P_, false>);
-#define REWL_TREE_P(W_, S_)                                                \
-    if (p.precision == REWL_FP64) { REWL_TREE_G(W_, S_, REWL_FP64) }       \
-    else { REWL_TREE_G(W_, S_, REWL_F32X2) }
-    if (p.wpr == 1) {
-        if (smt) { REWL_TREE_P(1, true) } else { REWL_TREE_P(1, false) }
-    } else {
-        if (smt) { REWL_TREE_P(2, true) } else { REWL_TREE_P(2, false) }
+    const bool wide = blocks_of(p.L).n > 1;
+#define REWL_TREE_G(S_, P_, R_, W_)                                   \
+    if (group == 32) return go(k_sweep_tree<S_, 32, P_, R_, W_>);     \
+    if (group == 16) return go(k_sweep_tree<S_, 16, P_, R_, W_>);     \
+    return go(k_sweep_tree<S_, 8, P_, R_, W_>);
+#define REWL_TREE_R(S_, P_)                                           \
+    if (p.lattice_reg) { REWL_TREE_G(S_, P_, true, false) }           \
+    if (wide) { REWL_TREE_G(S_, P_, false, true) }                    \
+    REWL_TREE_G(S_, P_, false, false)
+    if (p.precision == REWL_FP64) {
+        if (smt) { REWL_TREE_R(true, REWL_FP64) }
+        REWL_TREE_R(false, REWL_FP64)
     }
-#undef REWL_TREE_P
+    if (smt) { REWL_TREE_R(true, REWL_F32X2) }
+    REWL_TREE_R(false, REWL_F32X2)
+#undef REWL_TREE_R
 #undef REWL_TREE_G
 }
 

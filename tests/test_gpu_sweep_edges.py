@@ -1,0 +1,68 @@
+"""The warp sampler at the edges of its lattice blocks, groups and table
+placements, bit for bit against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import OracleConfig, OracleREWL
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1508_02748_gb300 as P
+    from paper_1508_02748_gb300 import build
+    build.build()
+    return P
+
+
+def _same(P, steps, tile, **kw):
+    o = OracleREWL(OracleConfig(**kw))
+    g = P.REWL(P.Config(**kw, **tile))
+    for n in steps:
+        o.sweep(n)
+        g.sweep(n)
+        so, spo = o.walkers()
+        sg, spg = g.walkers()
+        np.testing.assert_array_equal(sg[:, :3], so[:, :3])
+        np.testing.assert_array_equal(spg, spo)
+        lo, Ho, _ = o.tables()
+        lg, Hg = g.tables()
+        np.testing.assert_array_equal(Hg, Ho)
+        np.testing.assert_array_equal(lg, lo)
+    g.close()
+    o.close()
+
+
+# rows of one block (L <= 30 and L = 32), of two (31, 33-60) and of three
+# (61-64); 5 walkers: groups of 8 and 16 lanes leave idle ones in a warp;
+# launches shorter than a step, and ones that end in the middle of one
+@pytest.mark.parametrize("lanes", [32, 16, 8])
+@pytest.mark.parametrize("L", [7, 9, 29, 30, 31, 32, 34, 60, 61, 62])
+def test_lattice_blocks_and_idle_groups(P, L, lanes):
+    _same(P, (1, 2, 3, 4, 5, 6, 1500), dict(lanes_per_walker=lanes), L=L, walkers_per_window=5, seed=300 + L)
+
+
+# a grid with empty windows: their walkers' groups share warps with live ones
+@pytest.mark.parametrize("lanes,tables", [(16, 1), (16, 2), (8, 1), (8, 2)])
+def test_empty_windows_beside_live_ones(P, lanes, tables):
+    kw = dict(L=8, n_win_E=6, n_win_M=6, overlap_E=0.5, overlap_M=0.5, walkers_per_window=3, seed=17,
+              drive_budget=10**8)
+    _same(P, (7, 2000), dict(lanes_per_walker=lanes, table_mode=tables, walkers_per_block=2), **kw)
+
+
+def test_staged_window_at_the_shared_memory_limit(P):
+    """28,390 bins fit in a block's shared memory, their staged rows with the
+    entries around them do not: the run still goes, from global memory."""
+    kw = dict(L=13, n_win_E=2, overlap_E=0.98, walkers_per_window=1, seed=5)
+    _same(P, (3, 1200), dict(lanes_per_walker=32, table_mode=P.TABLES_STAGED), **kw)
+
+
+# narrow windows: staged rows are padded to 16 entries
+@pytest.mark.parametrize("lattice", [1, 2])
+def test_staged_narrow_rows(P, lattice):
+    kw = dict(L=4, n_win_M=4, overlap_M=0.5, walkers_per_window=3, seed=23, drive_budget=10**8)
+    _same(P, (5, 1700), dict(lanes_per_walker=32, table_mode=P.TABLES_STAGED, lattice_mode=lattice), **kw)
