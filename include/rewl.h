@@ -66,14 +66,16 @@ extern "C" {
 
 /* Where the warp sampler keeps a walker's screen and visit counts during a
  * launch (rewl_config.table_mode); every choice gives the same trajectory. */
-#define REWL_TABLES_AUTO 0      /* staged when the window's bins fit in shared memory, else global */
+#define REWL_TABLES_AUTO 0      /* staged when the windows of all walkers fit in the GPU's shared memory
+                                   at once, else global */
 #define REWL_TABLES_GLOBAL 1    /* global memory (L1-cached) */
 #define REWL_TABLES_STAGED 2    /* all of the walker's bins in shared memory for the launch (REWL_E_CUDA
                                    at launch when they do not fit) */
 
 /* How the warp sampler holds a walker's lattice during a launch
  * (rewl_config.lattice_mode); every choice gives the same trajectory. */
-#define REWL_LATTICE_AUTO 0     /* a register when N <= 64, else shared memory */
+#define REWL_LATTICE_AUTO 0     /* a register when N <= 64 and the tables are staged or a walker has 8
+                                   lanes, else shared memory */
 #define REWL_LATTICE_REGISTER 1 /* one 64-bit register per lane (N <= 64 only, else REWL_E_INVALID) */
 #define REWL_LATTICE_SHARED 2   /* one 32-bit word per row in shared memory (two for L > 32) */
 

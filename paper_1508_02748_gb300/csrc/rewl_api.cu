@@ -236,6 +236,45 @@ int max_pairs_of(const Dims &d)
     return best;
 }
 
+// How the warp sampler maps a run onto the GPU when `walkers` walkers (its
+// own, or those of all runs of a batch) share it; what the configuration
+// fixes stays.  Every choice gives the same chains.  Times are ms per 10^4
+// trials of every walker on a GB300.
+//   - Staged tables while all walkers fit on the GPU's shared memory at once:
+//     L = 8, 3 x 3 windows, staged against global: 36 walkers 0.43 / 0.57, 1350
+//     0.63 / 0.81; past that the staged walkers take turns: 1800 0.94 / 0.81.
+//   - Staged: 32 lanes up to one warp per SM sub-partition (450 walkers 0.43,
+//     16 lanes 0.49), then 16 (900: 0.53 against 0.49); more walkers make the
+//     step's instructions count, fewer its depth.
+//   - Global: 32 lanes while that is at most 16 warps an SM (L = 32, 2048
+//     walkers: 1.05, 16 lanes 1.28; 2560: 1.47 against 1.37), 16 lanes while
+//     that is at most the 18 warps an SM that the registers allow (5120: 16
+//     lanes 1.72, 8 lanes 2.31), then 8 (8192: 2.91 against 2.53).
+//   - A lattice of N <= 64 in a register beside staged tables and with 8 lanes
+//     (1.50 against 1.69); with global tables and more lanes its longer chain
+//     costs more than its loads save (0.57 against 0.69 at 32).
+void choose_tiling(rewl_t *h, long long walkers)
+{
+    constexpr long long kSMs = 152;
+    constexpr size_t kSmem = 227 * 1024, kPerBlock = 1024;
+    Params &p = h->p;
+    const rewl_config &c = h->cfg;
+    const bool small = p.N <= 64 && p.wpr == 1 && c.lattice_mode != REWL_LATTICE_SHARED;
+    const long long per_sm = (walkers + kSMs - 1) / kSMs;
+    const int staged_lanes = c.lanes_per_walker ? c.lanes_per_walker : walkers <= 4 * kSMs ? 32 : 16;
+    const int global_lanes = c.lanes_per_walker ? c.lanes_per_walker
+                           : walkers <= 16 * kSMs ? 32 : walkers <= 36 * kSMs ? 16 : 8;
+    p.lattice_reg = small ? 1 : 0;
+    const size_t gpw = (size_t)(32 / staged_lanes);
+    const size_t block = tree_smem_per_warp(p, true, staged_lanes) * gpw + kPerBlock;
+    const size_t blocks = (size_t)((per_sm + (long long)gpw - 1) / (long long)gpw);
+    if (p.sampler != REWL_SAMPLER_WARP) p.smt = 0;
+    else if (c.table_mode != REWL_TABLES_AUTO) p.smt = c.table_mode == REWL_TABLES_STAGED;
+    else p.smt = block * (blocks ? blocks : 1) <= kSmem + kPerBlock;
+    p.group = p.smt ? staged_lanes : global_lanes;
+    if (c.lattice_mode == REWL_LATTICE_AUTO && !p.smt && p.group != 8) p.lattice_reg = 0;
+}
+
 int sync(rewl_t *h)
 {
     CK(h, cudaStreamSynchronize(h->stream));
@@ -373,8 +412,6 @@ int create_impl(const rewl_config *cfg, const uint8_t *host_init_spins, void *d_
     p.wE = d.wE; p.wM = d.wM; p.T = d.T; p.tstride = d.tstride;
     p.precision = cfg->precision;
     p.sampler = cfg->sampler;
-    // stage the tables in shared memory when a warp's share stays small
-    p.smt = 0;
     p.key0 = (uint32_t)cfg->seed; p.key1 = (uint32_t)(cfg->seed >> 32);
     p.divL = (uint32_t)((0x100000000ull + (unsigned long long)d.L - 1) / (unsigned long long)d.L);
     p.lnf_final = cfg->lnf_final; p.lnf_factor = cfg->lnf_factor;
@@ -440,17 +477,7 @@ int create_impl(const rewl_config *cfg, const uint8_t *host_init_spins, void *d_
             n_active += any ? 1 : 0;
         }
     p.n_active_walkers = n_active * d.W;
-    // lanes per walker: a whole warp while walkers are few, packed groups when
-    // the walkers alone can fill the GPU
-    if (cfg->lanes_per_walker) p.group = cfg->lanes_per_walker;
-    else p.group = p.n_active_walkers <= 1216 ? 32 : (p.n_active_walkers <= 2432 ? 16 : 8);
-    p.lattice_reg = (cfg->lattice_mode == REWL_LATTICE_SHARED || d.N > 64 || d.wpr != 1) ? 0 : 1;
-    // where the warp sampler keeps S and H during a launch: staged in shared
-    // memory when a warp's share stays small, else global memory
-    if (cfg->table_mode == REWL_TABLES_STAGED) p.smt = 1;
-    else if (cfg->table_mode == REWL_TABLES_GLOBAL) p.smt = 0;
-    else p.smt = tree_smem_per_warp(p, true, p.group) * (size_t)(32 / p.group) <= 100 * 1024 ? 1 : 0;
-    if (p.sampler != REWL_SAMPLER_WARP) p.smt = 0;
+    choose_tiling(h, p.n_active_walkers);
     h->first_active = -1;
     for (int win = 0; win < d.nwin && h->first_active < 0; ++win)
         if (active[win]) h->first_active = win * d.W;
@@ -1096,17 +1123,22 @@ extern "C" int rewl_batch_create(rewl_t *const *runs, int n, void *stream, rewl_
             return fail(nullptr, REWL_E_CUDA, "batch: stream: %s", cudaGetErrorString(e));
         }
     // Capture: fork from the batch stream, K cycles of each run on its own
-    // stream, join back.  The runs' own streams are swapped for the capture.
+    // stream, join back.  The runs' own streams and tilings are swapped for the
+    // capture.
     cudaGraph_t g = nullptr;
     if ((e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) {
         batch_free(b);
         return fail(nullptr, REWL_E_CUDA, "batch: begin capture: %s", cudaGetErrorString(e));
     }
     cudaError_t qe = cudaEventRecord(b->events[n], b->stream);
+    long long walkers = 0;               // of all the runs: they share the GPU
+    for (rewl_t *h : b->runs) walkers += h->p.n_active_walkers;
     for (int i = 0; i < n && qe == cudaSuccess; ++i) {
         rewl_t *h = b->runs[i];
         cudaStream_t own = h->stream;
+        const Params alone = h->p;
         h->stream = b->streams[i];
+        choose_tiling(h, walkers);
         qe = cudaStreamWaitEvent(h->stream, b->events[n], 0);
         const unsigned long long ce = (unsigned long long)h->cfg.check_every;
         for (unsigned long long c = 0; c < b->k && qe == cudaSuccess; ++c)
@@ -1114,6 +1146,7 @@ extern "C" int rewl_batch_create(rewl_t *const *runs, int n, void *stream, rewl_
         if (qe == cudaSuccess) qe = cudaEventRecord(b->events[i], h->stream);
         if (qe == cudaSuccess) qe = cudaStreamWaitEvent(b->stream, b->events[i], 0);
         h->stream = own;
+        h->p = alone;
     }
     e = cudaStreamEndCapture(b->stream, &g);
     if (qe != cudaSuccess || e != cudaSuccess) {

@@ -66,3 +66,29 @@ def test_staged_window_at_the_shared_memory_limit(P):
 def test_staged_narrow_rows(P, lattice):
     kw = dict(L=4, n_win_M=4, overlap_M=0.5, walkers_per_window=3, seed=23, drive_budget=10**8)
     _same(P, (5, 1700), dict(lanes_per_walker=32, table_mode=P.TABLES_STAGED, lattice_mode=lattice), **kw)
+
+
+# either side of each line of the automatic tiling (staged or global tables,
+# 32, 16 or 8 lanes, lattice in a register or not), against the thread sampler
+@pytest.mark.parametrize("L,nE,nM,W", [(4, 1, 1, 608), (4, 1, 1, 609), (8, 3, 3, 185), (8, 3, 3, 186), (8, 3, 3, 271),
+                                       (6, 3, 2, 912), (6, 3, 2, 913), (12, 2, 1, 76), (12, 2, 1, 77)])
+def test_automatic_tiling(P, L, nE, nM, W):
+    kw = dict(L=L, n_win_E=nE, n_win_M=nM, walkers_per_window=W, seed=40 + L, exchange_interval=700)
+    a, b = P.REWL(P.Config(**kw)), P.REWL(P.Config(sampler=P.SAMPLER_THREAD, **kw))
+    sa, sb = a.run_cycles(3), b.run_cycles(3)
+    assert sa == sb and a.digest() == b.digest()
+    np.testing.assert_array_equal(a.walkers()[1], b.walkers()[1])
+
+
+# in a batch the runs' walkers share the GPU, so the tiling goes by their sum
+def test_batch_tiling_keeps_the_chains(P):
+    kws = [dict(L=L, n_win_E=3, n_win_M=2, walkers_per_window=w, seed=s, exchange_interval=900)
+           for L, w, s in ((8, 300, 1), (8, 200, 2), (16, 70, 3))]
+    alone, together = [[P.REWL(P.Config(**kw)) for kw in kws] for _ in range(2)]
+    P.Batch(together).run_cycles(4)
+    for a, t in zip(alone, together):
+        a.run_cycles(4)
+        assert a.digest() == t.digest()
+        np.testing.assert_array_equal(a.walkers()[0], t.walkers()[0])
+        a.run_cycles(2), t.run_cycles(2)                 # and each goes on alone
+        assert a.digest() == t.digest()
