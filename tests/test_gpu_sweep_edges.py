@@ -92,3 +92,36 @@ def test_batch_tiling_keeps_the_chains(P):
         np.testing.assert_array_equal(a.walkers()[0], t.walkers()[0])
         a.run_cycles(2), t.run_cycles(2)                 # and each goes on alone
         assert a.digest() == t.digest()
+
+
+# the digest's chunks and vector tails, and a flatness check split over a
+# cluster's blocks (windows of 30,276 bins and few walkers) or not: the digest
+# from its definition on the host, the verdicts from the 80% rule
+@pytest.mark.parametrize("L,nE,W,prec", [(4, 1, 2, 0), (13, 1, 3, 0), (13, 1, 3, 1), (13, 1, 700, 1), (6, 3, 5, 0),
+                                         (13, 1, 2, 2)])
+def test_digest_and_flatness(P, L, nE, W, prec):
+    r = P.REWL(P.Config(L=L, n_win_E=nE, walkers_per_window=W, seed=3, precision=prec, exchange_interval=500))
+    r.run_cycles(2)
+    lng, H = r.tables()
+    rng = np.random.default_rng(L + W)
+    n = H.size // r.n_walkers
+    for w in range(r.n_walkers):       # either side of the line
+        H[w * n:(w + 1) * n] = np.where(rng.random(n) < 0.7, rng.integers(66 + w % 2, 101, n), -1)
+    lng = np.round(lng * 256) / 256
+    r.set_tables(lng, H)
+    lng, H = r.tables()
+
+    def mix(z):
+        z = (z ^ (z >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+        z = (z ^ (z >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+        return z ^ (z >> np.uint64(31))
+
+    with np.errstate(over="ignore"):
+        i = np.arange(H.size, dtype=np.uint64)
+        h = H.astype(np.uint32).astype(np.uint64)
+        want = int((mix(lng.view(np.uint64) ^ mix(i)) + mix(h + np.uint64(0x9E3779B97F4A7C15) * i)).sum(dtype=np.uint64))
+    assert r.digest() == want
+    r.check()
+    Hw = H.reshape(r.n_walkers, n)
+    flat = [int(x[x >= 0].min()) * (x >= 0).sum() * 10**6 >= 800000 * int(x[x >= 0].sum()) for x in Hw]
+    np.testing.assert_array_equal(r.walkers(spins=False)[0][:, 3], np.array(flat, dtype=np.int64))
