@@ -12,6 +12,8 @@
 //   PERM  (x, pair, i, 4)         Fisher-Yates draw i of exchange sweep x
 //   EXCH  (x, pair, k, 5)         acceptance draw of the k-th pair
 // pair = 2 * (lower window) + axis.
+#include <cooperative_groups.h>
+
 #include "rewl_tab.cuh"
 
 namespace rewl {
@@ -387,10 +389,19 @@ cudaError_t launch_sweep_walker(const Params &p, int w, uint64_t ntrials, cudaSt
 // X, Y the configurations of walkers i (lower) and j (upper) before the swap,
 // each g the walker's own table.  On acceptance the lattices and bins swap;
 // no g or H is updated.
-__global__ void k_exchange(Params p)
+//
+// Bounded by latency: few blocks, each a chain of draws, table reads and
+// swaps.  The permutation's draws are made by all threads at once and only its
+// W - 1 swaps of indices by one, and the accepted pairs' lattice words are
+// swapped by all threads (a word of adjacent walkers is adjacent).  Per sweep,
+// before (draws by one thread, each pair's words one after the other by one
+// thread) -> after: L = 32, 32 walkers a window 19 -> 10 us; L = 64, 16 walkers 49
+// -> 14; L = 33, 5 walkers 25 -> 9.
+__global__ void __launch_bounds__(256) k_exchange(Params p)
 {
-    extern __shared__ int perm[];
-    __shared__ unsigned long long s_att, s_acc;
+    extern __shared__ int perm[];              // W partners, then W draws / accepted flags
+    int *const work = perm + p.W;
+    __shared__ unsigned s_att, s_acc;
     if (p.st->done) return;
     const unsigned long long xs = p.st->xstep;
     const int phase = (int)(xs & 3ull), axis = phase >> 1, parity = phase & 1;
@@ -406,82 +417,107 @@ __global__ void k_exchange(Params p)
     if (!p.active[A] || !p.active[B]) return;
     const int W = p.W;
     const uint32_t pair = (uint32_t)(2 * A + axis);
+    for (int i = threadIdx.x; i < W; i += blockDim.x) {
+        perm[i] = i;
+        if (i) work[i] = (int)__umulhi(philox10((uint32_t)xs, pair, (uint32_t)i, TAG_PERM, p.key0, p.key1).x, (uint32_t)(i + 1));
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 0; k < W; ++k) perm[k] = k;
         for (int i = W - 1; i >= 1; --i) {
-            const u32x4 r = philox10((uint32_t)xs, pair, (uint32_t)i, TAG_PERM, p.key0, p.key1);
-            const int j = (int)__umulhi(r.x, (uint32_t)(i + 1));
+            const int j = work[i];
             const int tmp = perm[i]; perm[i] = perm[j]; perm[j] = tmp;
         }
-        s_att = 0ull; s_acc = 0ull;
+        s_att = 0u; s_acc = 0u;
     }
     __syncthreads();
     const int4 RA = p.rect[A], RB = p.rect[B];
+    const double lnf = p.st->lnf;
     for (int k = threadIdx.x; k < W; k += blockDim.x) {
         const int wi = A * W + k, wj = B * W + perm[k];
         const int eX = p.we[wi], mX = p.wm[wi], eY = p.we[wj], mY = p.wm[wj];
         const bool xinB = eX >= RB.x && eX <= RB.y && mX >= RB.z && mX <= RB.w;
         const bool yinA = eY >= RA.x && eY <= RA.y && mY >= RA.z && mY <= RA.w;
-        if (!xinB || !yinA) continue;
-        const size_t bi = (size_t)wi * p.tstride, bj = (size_t)wj * p.tstride;
-        const double lnf = p.st->lnf;
-        const double giX = lng_read(p, bi + (size_t)(eX - RA.x) * p.wM + (mX - RA.z), lnf);
-        const double giY = lng_read(p, bi + (size_t)(eY - RA.x) * p.wM + (mY - RA.z), lnf);
-        const double gjY = lng_read(p, bj + (size_t)(eY - RB.x) * p.wM + (mY - RB.z), lnf);
-        const double gjX = lng_read(p, bj + (size_t)(eX - RB.x) * p.wM + (mX - RB.z), lnf);
-        const double lnP = (giX - giY) + (gjY - gjX);
-        const u32x4 r = philox10((uint32_t)xs, pair, (uint32_t)k, TAG_EXCH, p.key0, p.key1);
-        atomicAdd(&s_att, 1ull);
-        if (lnP >= 0.0 || log(unit_open(r.x)) < lnP) {
-            for (int word = 0; word < p.nwords; ++word) {
-                uint32_t *pa = p.spins + (size_t)word * p.nwalk + wi;
-                uint32_t *pb = p.spins + (size_t)word * p.nwalk + wj;
-                const uint32_t tmp = *pa; *pa = *pb; *pb = tmp;
+        bool accept = false;
+        if (xinB && yinA) {
+            const size_t bi = (size_t)wi * p.tstride, bj = (size_t)wj * p.tstride;
+            const double giX = lng_read(p, bi + (size_t)(eX - RA.x) * p.wM + (mX - RA.z), lnf);
+            const double giY = lng_read(p, bi + (size_t)(eY - RA.x) * p.wM + (mY - RA.z), lnf);
+            const double gjY = lng_read(p, bj + (size_t)(eY - RB.x) * p.wM + (mY - RB.z), lnf);
+            const double gjX = lng_read(p, bj + (size_t)(eX - RB.x) * p.wM + (mX - RB.z), lnf);
+            const double lnP = (giX - giY) + (gjY - gjX);
+            const u32x4 r = philox10((uint32_t)xs, pair, (uint32_t)k, TAG_EXCH, p.key0, p.key1);
+            atomicAdd(&s_att, 1u);
+            accept = lnP >= 0.0 || log(unit_open(r.x)) < lnP;
+            if (accept) {
+                p.we[wi] = eY; p.wm[wi] = mY;
+                p.we[wj] = eX; p.wm[wj] = mX;
+                atomicAdd(&s_acc, 1u);
             }
-            p.we[wi] = eY; p.wm[wi] = mY;
-            p.we[wj] = eX; p.wm[wj] = mX;
-            atomicAdd(&s_acc, 1ull);
         }
+        work[k] = accept;
     }
     __syncthreads();
+    for (int i = threadIdx.x; i < W * p.nwords; i += blockDim.x) {
+        const int word = i / W, k = i - word * W;
+        if (!work[k]) continue;
+        uint32_t *pa = p.spins + (size_t)word * p.nwalk + A * W + k;
+        uint32_t *pb = p.spins + (size_t)word * p.nwalk + B * W + perm[k];
+        const uint32_t tmp = *pa; *pa = *pb; *pb = tmp;
+    }
     if (threadIdx.x == 0 && s_att) {
-        atomicAdd(&p.st->exch_attempts, s_att);
-        atomicAdd(&p.st->exch_accepts, s_acc);
+        atomicAdd(&p.st->exch_attempts, (unsigned long long)s_att);
+        atomicAdd(&p.st->exch_accepts, (unsigned long long)s_acc);
     }
 }
 
 cudaError_t launch_exchange(const Params &p, int max_pairs, cudaStream_t s)
 {
     if (max_pairs <= 0) return cudaSuccess;
-    const int threads = p.W <= 32 ? 32 : (p.W <= 128 ? 128 : 256);
-    k_exchange<<<max_pairs, threads, (size_t)p.W * sizeof(int), s>>>(p);
+    const long long tasks = (long long)p.W * p.nwords;
+    const int threads = tasks <= 64 ? 64 : tasks <= 128 ? 128 : 256;
+    k_exchange<<<max_pairs, threads, 2 * (size_t)p.W * sizeof(int), s>>>(p);
     return cudaGetLastError();
 }
 
 // --------------------------------------------------------------- flat ----
 
-// One block per walker: over visited bins (H >= 0), n_seen, sum H and min H;
-// flat iff min H * n_seen * 10^6 >= round(flatness * 10^6) * sum H (the 80%
-// rule of Sec. 3 in exact integers).
+// One cluster of blocks per walker: over visited bins (H >= 0), n_seen, sum H
+// and min H; flat iff min H * n_seen * 10^6 >= round(flatness * 10^6) * sum H
+// (the 80% rule of Sec. 3 in exact integers).
+//
+// Bounded by HBM (4 bytes a bin) once enough blocks read: one block a walker
+// leaves most of the chip idle below some 600 walkers (L = 33, 105 walkers of
+// 317,000 bins: 89 us, 1.5 TB/s), so a walker's bins are split over up to 8
+// blocks of a cluster, whose parts meet in the first one's shared memory
+// (89 -> 29 us; 2048 walkers at L = 32 stay at one block each, 161 us, 6.4 TB/s).
+struct FlatPart {
+    long long cnt, sum;
+    int mn;
+};
+
+template <bool SPLIT>
 __global__ void __launch_bounds__(256) k_flat(Params p)
 {
     if (p.st->done) return;
-    const int w = blockIdx.x;
-    if (!p.active[w / p.W]) return;
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cl = cg::this_cluster();
+    const int rank = SPLIT ? (int)cl.block_rank() : 0, parts = SPLIT ? (int)cl.num_blocks() : 1;
+    const int w = (int)blockIdx.x / parts;
+    if (!p.active[w / p.W]) return;            // (the whole cluster)
     const int32_t *H = p.H + (size_t)w * p.tstride;
     long long cnt = 0, sum = 0;
     int mn = 0x7FFFFFFF;
     const int T = p.T;
     const int T4 = T & ~3;
     const int4 *H4 = reinterpret_cast<const int4 *>(H);
-    for (int i = threadIdx.x; i < T4 / 4; i += blockDim.x) {
+    for (int i = rank * 256 + (int)threadIdx.x; i < T4 / 4; i += parts * 256) {
         const int4 v = H4[i];
         if (v.x >= 0) { ++cnt; sum += v.x; mn = min(mn, v.x); }
         if (v.y >= 0) { ++cnt; sum += v.y; mn = min(mn, v.y); }
         if (v.z >= 0) { ++cnt; sum += v.z; mn = min(mn, v.z); }
         if (v.w >= 0) { ++cnt; sum += v.w; mn = min(mn, v.w); }
     }
-    for (int i = T4 + threadIdx.x; i < T; i += blockDim.x) {
+    for (int i = T4 + rank * 256 + (int)threadIdx.x; i < T; i += parts * 256) {
         const int v = H[i];
         if (v >= 0) { ++cnt; sum += v; mn = min(mn, v); }
     }
@@ -490,14 +526,16 @@ __global__ void __launch_bounds__(256) k_flat(Params p)
         sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
         mn = min(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
     }
-    __shared__ long long s_cnt[8], s_sum[8];
-    __shared__ int s_mn[8];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) { s_cnt[wid] = cnt; s_sum[wid] = sum; s_mn[wid] = mn; }
+    __shared__ FlatPart s_warp[8], s_block[8];
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = {cnt, sum, mn};
     __syncthreads();
     if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        for (int k = 1; k < nw; ++k) { cnt += s_cnt[k]; sum += s_sum[k]; mn = min(mn, s_mn[k]); }
+        for (int k = 1; k < 8; ++k) { cnt += s_warp[k].cnt; sum += s_warp[k].sum; mn = min(mn, s_warp[k].mn); }
+        if constexpr (SPLIT) *cl.map_shared_rank(&s_block[rank], 0) = {cnt, sum, mn};
+    }
+    if constexpr (SPLIT) cl.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        for (int k = 1; k < parts; ++k) { cnt += s_block[k].cnt; sum += s_block[k].sum; mn = min(mn, s_block[k].mn); }
         const int flat = cnt > 0 && (long long)mn * cnt * 1000000ll >= p.flat_q * sum;
         p.wflat[w] = flat;
         if (flat) atomicAdd(&p.st->nflat, 1);
@@ -506,8 +544,25 @@ __global__ void __launch_bounds__(256) k_flat(Params p)
 
 cudaError_t launch_flat(const Params &p, cudaStream_t s)
 {
-    k_flat<<<p.nwalk, 256, 0, s>>>(p);
-    return cudaGetLastError();
+    // blocks a walker: until 8 blocks an SM or until a block has 8192 bins
+    int parts = 1;
+    while (parts < 8 && (long long)p.nwalk * parts < 152 * 4 && p.T / (2 * parts) >= 8192) parts *= 2;
+    if (parts == 1) {
+        k_flat<false><<<p.nwalk, 256, 0, s>>>(p);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)p.nwalk * parts);
+    lc.blockDim = dim3(256);
+    lc.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = parts;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    lc.attrs = &at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, k_flat<true>, p);
 }
 
 // ------------------------------------------------------------- decide ----
