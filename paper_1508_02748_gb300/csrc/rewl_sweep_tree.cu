@@ -54,15 +54,15 @@
 //     pair converts exactly) and equals the sequential additions whenever
 //     ln f = 2^-k and the values stay within 53 (pair: 48) bits;
 //   - the float screen is decided only outside a margin that bounds its
-//     error.  With x = S + H ln f of a bin in float, t = ln u - (x_c - x_n +
-//     v ln f), v the difference of the step's visits, errs by at most
+//     error.  With x = S + H ln f of a bin in float, t = (ln u + v ln f) - (x_c
+//     - x_n), v the difference of the step's visits, errs by at most
 //       2^-24 |S| + 2^-24 (|x| + |S|) + 2^-24 |x| per bin (the screen, the
 //         count converted to float, the fma),
 //       2^-24 (|x_c| + |x_n|) (their difference),
+//       2^-24 (|t| + |x_c| + |x_n|) + 2^-24 |t| (ln u + v ln f, which is t and
+//         the difference together, and the last subtraction), and
 //       0.51 2^-20 (|ln u| + 1) (u rounds with relative error below 2^-23;
-//         __logf errs by at most 2^-21.41 in [1/2, 1] and 3 ulp below), and
-//       2^-22 |t| (the last fma and subtraction, where v ln f or t is the
-//         largest term),
+//         __logf errs by at most 2^-21.41 in [1/2, 1] and 3 ulp below),
 //     below 0.51 M + 2^-22 |t| with M = 2^-20 (|S_c| + |x_c| + |S_n| + |x_n| +
 //     |ln u|) + 2^-20, so the sign of t is the decision whenever |t| > M.
 //     Otherwise the decision is re-taken from the exact difference: against
@@ -76,7 +76,7 @@
 // comparisons, the leaf by shuffle instead of a mailbox, the trial read a step
 // ahead and near-ties looked at on the path alone took 266-302 instructions a
 // step to 150.  Sampling launches of 10^4 trials per walker, GB300, 2070 MHz,
-// before -> after: L = 8 (36 walkers, 32 lanes, staged) 0.72 -> 0.41 ms; L = 16
+// before -> after: L = 8 (36 walkers, 32 lanes, staged) 0.72 -> 0.37 ms; L = 16
 // (256 walkers, 32 lanes) 0.95 -> 0.64 ms; L = 32 (2048 walkers, 32 lanes) 1.64
 // -> 1.05 ms; L = 64 (3904 walkers, 16 lanes) 2.71 -> 1.60 ms.
 // Tried and slower: the visits of recent bins in a shared-memory cache (L1
@@ -131,11 +131,12 @@ struct RingEntry {
     uint32_t f;    // shared lattice, one block a row: mask of the site's bit(s) in its word
                    // shared lattice, several blocks: the site's copy in another block: 1 | its bit << 1 |
                    //   its word minus the site's, plus 2, << 6 (0: none)
-                   // register lattice: the site
     float lnu;     // ln u in float
 };
 static_assert(sizeof(RingEntry) == 16, "one vector load per trial");
 constexpr size_t RING_BYTES = (RING + RING_TAIL) * sizeof(RingEntry);
+// Register lattice: each trial's site as a 64-bit mask, beside the ring.
+constexpr size_t BITS_BYTES = (RING + RING_TAIL) * sizeof(uint2);
 
 // Eq. 1 decided from the exact values (near-ties of the float screen on the
 // true path only).
@@ -193,6 +194,7 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
 
     unsigned char *base = smem_raw + (size_t)slot * smem_per_walker;
     RingEntry *ring = reinterpret_cast<RingEntry *>(base);
+    uint2 *bits = reinterpret_cast<uint2 *>(base + RING_BYTES);        // REG
     uint32_t *lat = reinterpret_cast<uint32_t *>(base + RING_BYTES);   // nlat words and G that take the idle lanes' flips
     const int L = p.L;
     const Blocks bk = blocks_of(L);
@@ -208,7 +210,7 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
     const int wM = p.wM;
     const int ld = staged_ld(wM);
     const int nstaged = (p.wE + 4) * ld;
-    int2 *tab = reinterpret_cast<int2 *>(base + RING_BYTES + (REG ? 0 : ((nlat + G) * 4 + 15) & ~15));
+    int2 *tab = reinterpret_cast<int2 *>(base + RING_BYTES + (REG ? BITS_BYTES : ((nlat + G) * 4 + 15) & ~15));
     if constexpr (SMT) {
         #pragma unroll 4
         for (int k = gl; k < nstaged; k += G) {
@@ -349,13 +351,16 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
                     const uint32_t j = site - i * (uint32_t)L;
                     const uint32_t iu = i == 0 ? L - 1 : i - 1, id = i == (uint32_t)L - 1 ? 0 : i + 1;
                     RingEntry en;
+                    uint2 own = make_uint2(0u, 0u);
                     if (REG) {
                         const uint32_t jl = j == 0 ? L - 1 : j - 1, jr = j == (uint32_t)L - 1 ? 0 : j + 1;
                         const unsigned long long nb = (1ull << (iu * L + j)) | (1ull << (id * L + j))
                                                     | (1ull << (i * L + jl)) | (1ull << (i * L + jr));
                         en.a = (uint32_t)nb;
                         en.b = (uint32_t)(nb >> 32);
-                        en.f = site;
+                        en.f = 0;
+                        const unsigned long long o = 1ull << site;
+                        own = make_uint2((uint32_t)o, (uint32_t)(o >> 32));
                     } else {
                         en.b = site << 20;
                         if (WIDE) {
@@ -378,7 +383,11 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
                     en.lnu = __logf(__fmaf_rn(__uint2float_rn(xu), 0x1p-32f, 0x1p-33f));
                     const unsigned at = (unsigned)(2 * c + hh) & RMASK;
                     ring[at] = en;
-                    if (at < RING_TAIL) ring[at + RING] = en;
+                    if (REG) bits[at] = own;
+                    if (at < RING_TAIL) {
+                        ring[at + RING] = en;
+                        if (REG) bits[at + RING] = own;
+                    }
                 }
             }
             __syncwarp();
@@ -423,17 +432,19 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
         // a step ahead: the lane's trial and, REG, the sites its history flips
         RingEntry nxt;
         uint32_t nlo = 0, nhi = 0;
+        uint2 nbit = make_uint2(0u, 0u);
         auto ahead = [&](unsigned at) {
-            const RingEntry *now = ring + (at & RMASK);
-            nxt = now[dl];
+            const unsigned now = at & RMASK;
+            nxt = ring[now + dl];
             if (REG) {
                 nlo = nhi = 0;
                 #pragma unroll
                 for (int k = 0; k < DEPTH; ++k) {
-                    const unsigned long long b = 1ull << now[k].f;
-                    nlo ^= (uint32_t)b & flip[k];
-                    nhi ^= (uint32_t)(b >> 32) & flip[k];
+                    const uint2 b = bits[now + k];
+                    nlo ^= b.x & flip[k];
+                    nhi ^= b.y & flip[k];
                 }
+                nbit = bits[now + dl];
             }
         };
         ahead(r0 + u);
@@ -446,9 +457,8 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
         if (REG) {
             hlo = lo ^ nlo;
             hhi = hi ^ nhi;
-            const unsigned long long o = 1ull << me.f;
-            olo = (uint32_t)o;
-            ohi = (uint32_t)(o >> 32);
+            olo = nbit.x;
+            ohi = nbit.y;
             const bool sup = ((hlo & olo) | (hhi & ohi)) != 0u;
             pk = (__popc(hlo & me.a) + __popc(hhi & me.b)) * (sup ? mvA : -mvA) + (sup ? -mvB : mvB);
         } else {
@@ -507,7 +517,7 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
             mc = __shfl_sync(FULL, mn, src[0]);
         }
         ahead(r0 + u + DEPTH + 1);
-        const float t32 = __fsub_rn(me.lnu, __fmaf_rn(__int2float_rn(vcur - vnew), lnf32, __fsub_rn(xc, xn)));
+        const float t32 = __fsub_rn(__fmaf_rn(__int2float_rn(vnew - vcur), lnf32, me.lnu), __fsub_rn(xc, xn));
         const float M = __fmaf_rn(mc + mn + fabsf(me.lnu), 0x1p-20f, 0x1p-20f);
         bool acc = live && t32 < 0.0f;
         bool near = live && !(fabsf(t32) > M);      // (not a number counts as near)
@@ -532,7 +542,8 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
             path = __shfl_sync(FULL, acc ? hacc : hist, leaf);   // bit k: trial k accepted
         };
         follow();
-        while (pm & nearb) {              // near-ties on the path are decided exactly
+        while (pm & nearb) {
+              // near-ties on the path are decided exactly
             if (onp && near) {
                 unsigned ib, jb;          // the bins' entries in the window's table
                 int hc;
@@ -556,7 +567,7 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
         // ---- commit: the visits of the path's bins are written: the count a bin
         // had, plus its earlier visits in the step, plus those until the path
         // leaves it.  A bin the path comes back to is written again with the
-        // larger count; the stores of such bins are ordered by rank.
+        // larger count; global stores of such bins are ordered by rank.
         P0 = Pa;
         if (REG) {
             lo = lo2;
@@ -569,16 +580,20 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
             atomicXor(flip ? word : own, WIDE ? 2u << (me.a & 31u) : me.f);
             if (WIDE) atomicXor(flip && (me.f & 1u) ? word + (int)(me.f >> 6) - 2 : own, 1u << ((me.f >> 1) & 31u));
         }
-        const int stay = __ffs((path | end) >> later) - (node ? 0 : 1);
+        const unsigned ahead_of = (path | end) >> later;
+        const int stay = __popc(ahead_of ^ (ahead_of - 1u)) - (node ? 0 : 1);   // trials up to its lowest bit
         const bool st = node ? onp && acc : first && stay > 0;
         const int val = hn + vnew + stay;
         if (st) err |= val;
-        #pragma unroll
-        for (int k = 0; k < (DEPTH >= 4 ? 3 : 2); ++k) {
-            if (k) __syncwarp();
-            if (st && rank == k) {
-                if constexpr (SMT) tab[nu].y = val;
-                else gH[nu] = val;
+        if constexpr (SMT) {
+            // (visits only grow: the larger count stays, in whatever order; lanes
+            // without a bin to write go to an entry outside the window)
+            atomicMax(&tab[st ? nu : (unsigned)gl].y, st ? val : -1);
+        } else {
+            #pragma unroll
+            for (int k = 0; k < (DEPTH >= 4 ? 3 : 2); ++k) {
+                if (k) __syncwarp();
+                if (st && rank == k) gH[nu] = val;
             }
         }
         __syncwarp();
@@ -623,8 +638,8 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
 // S and H (8 bytes per entry).
 size_t tree_smem_per_warp(const Params &p, bool smt, int group)
 {
-    const size_t nlat = p.lattice_reg ? 0 : (size_t)p.L * blocks_of(p.L).n + group;
-    size_t b = RING_BYTES + ((nlat * 4 + 15) & ~(size_t)15);
+    const size_t nlat = (size_t)p.L * blocks_of(p.L).n + group;
+    size_t b = RING_BYTES + (p.lattice_reg ? BITS_BYTES : (nlat * 4 + 15) & ~(size_t)15);
     if (smt) b += (size_t)(p.wE + 4) * staged_ld(p.wM) * 8;
     return (b + 15) & ~(size_t)15;
 }
@@ -645,8 +660,10 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
         smt = false;
     const size_t per = tree_smem_per_warp(p, smt, group);
     // one warp a block: blocks of several warps leave when their last walker
-    // does (16 lanes, L = 16: 0.90 ms at 1 warp, 1.00 at 4; 32 lanes: the same)
-    if (warps <= 0) warps = 1;
+    // does (16 lanes, L = 16: 0.90 ms at 1 warp, 1.00 at 4; 32 lanes: the same);
+    // and many walkers' blocks of four 8-lane groups do not all become resident
+    // (10,752 walkers at L = 32: 4.28 ms, 2.77 at two warps)
+    if (warps <= 0) warps = group == 8 ? 2 : 1;
     // no more warps per block than the shared memory of one block holds
     while (warps > 1 && per * (size_t)gpw * warps > max_smem) --warps;
     if (per * (size_t)gpw * warps > max_smem) return cudaErrorInvalidValue;
