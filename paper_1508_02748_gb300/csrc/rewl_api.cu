@@ -121,7 +121,7 @@ bool is_pow2(double x)
 
 struct Layout {
     size_t st, rect, active, spins, we, wm, wt, wflat, lng, H, scr;
-    size_t piece, off, GE, eshift, efrom, eto, ematch, rowok, F, mshift, mfrom, mto, mmatch, J, red, marg, gbuf;
+    size_t piece, off, GE, eshift, efrom, eto, ematch, rowok, F, mshift, mfrom, mto, mmatch, J, red, marg;
     size_t eslice, mslice;
     size_t jk_ref, jk_sum, jk_sq, jk_mean, jk_err;
     size_t fail, total;
@@ -211,7 +211,7 @@ Layout layout_of(const Dims &d)
     L.J = take(std::max(8 * B * B, (size_t)d.nwalk * d.N));
     L.red = take(8 * 2048);
     L.marg = take(8 * B);
-    L.gbuf = take(8 * 2 * B * (size_t)d.nM);
+    take(8 * 2 * B * (size_t)d.nM);          // spare: the workspace size stays what callers know
     L.eslice = take(8 * (size_t)d.nwin * d.wM);
     L.mslice = take(8 * (size_t)d.nM * B);
     L.jk_ref = take(8 * B * B);
@@ -448,7 +448,6 @@ int create_impl(const rewl_config *cfg, const uint8_t *host_init_spins, void *d_
     j.J = (double *)(base + lay.J);
     j.red = (double *)(base + lay.red);
     j.marg = (double *)(base + lay.marg);
-    j.gbuf = (double *)(base + lay.gbuf);
     j.eslice = (double *)(base + lay.eslice);
     j.mslice = (double *)(base + lay.mslice);
     j.jk_ref = (double *)(base + lay.jk_ref);
@@ -1001,19 +1000,25 @@ extern "C" int rewl_get_lng_jackknife(rewl_t *h, int what, double *host_mean, do
     if (needed) *needed = n;
     if (p0.W < 2) return fail(h, REWL_E_INVALID, "the jackknife needs at least two walkers per window");
     if (!host_mean || !host_err || capacity < n) return fail(h, REWL_E_CAPACITY, "need %zu entries", n);
+    // The replicates are queued one behind the other; the first one whose join
+    // fails leaves its number and code in the word that is read at the end.
     Params p = p0;
+    CK(h, cudaMemsetAsync(h->d_fail, 0, sizeof(int32_t), h->stream));
     for (int k = 0; k < p.W; ++k) {
         p.join_exclude = k;
         CK(h, cudaMemsetAsync(&p.st->join_error, 0, sizeof(int32_t), h->stream));
         CK(h, launch_join(p, h->j, h->stream));
         if (what == REWL_LNG_MARGINAL_E) CK(h, launch_marginal_e(p, h->j, h->stream));
-        CK(h, launch_jk_accum(h->j, what == REWL_LNG_JOINED ? h->j.J : h->j.marg, n, k, h->stream));
-        DevState ds;
-        const int rc = read_state(h, &ds);
-        if (rc) return rc;
-        if (ds.join_error) return fail(h, REWL_E_JOIN, "jackknife replicate %d: join failed (code %d)", k, ds.join_error);
+        CK(h, launch_jk_accum(p, h->j, what == REWL_LNG_JOINED ? h->j.J : h->j.marg, n, k, h->d_fail, h->stream));
     }
     CK(h, launch_jk_final(h->j, h->jk_mean, h->jk_err, n, p.W, h->stream));
+    int32_t failed = 0;
+    CK(h, cudaMemcpyAsync(&failed, h->d_fail, sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
+    DevState ds;
+    const int rc = read_state(h, &ds);
+    if (rc) return rc;
+    if (failed)
+        return fail(h, REWL_E_JOIN, "jackknife replicate %d: join failed (code %d)", failed >> 8, failed & 0xFF);
     CK(h, cudaMemcpyAsync(host_mean, h->jk_mean, 8 * n, cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaMemcpyAsync(host_err, h->jk_err, 8 * n, cudaMemcpyDeviceToHost, h->stream));
     return sync(h);

@@ -124,7 +124,6 @@ struct JoinScratch {
     double *J;        // (N+1) x (N+1) joined table
     double *red;      // reduction scratch (>= 2 * 1024 doubles)
     double *marg;     // N+1 marginal output
-    double *gbuf;     // nM x 2 x (N+1) work space of the E matching chains
     double *eslice;   // nwin x wM: rule 1, shift of each M slice of each piece within its row
     double *mslice;   // nM x (N+1): rule 1, shift of each E slice of each row
     double *jk_ref, *jk_sum, *jk_sq;   // jackknife accumulators, (N+1)^2 each
@@ -151,7 +150,10 @@ cudaError_t launch_philox(const uint32_t *d_ctr, uint32_t k0, uint32_t k1, uint3
                           uint64_t n, cudaStream_t s);
 cudaError_t launch_join(const Params &p, const JoinScratch &j, cudaStream_t s);
 cudaError_t launch_marginal_e(const Params &p, const JoinScratch &j, cudaStream_t s);
-cudaError_t launch_jk_accum(const JoinScratch &j, const double *x, size_t n, int k, cudaStream_t s);
+// Adds replicate k; where its join failed and no earlier one's did, *fail
+// becomes k << 8 | code.
+cudaError_t launch_jk_accum(const Params &p, const JoinScratch &j, const double *x, size_t n, int k, int32_t *fail,
+                            cudaStream_t s);
 cudaError_t launch_jk_final(const JoinScratch &j, double *mean, double *err, size_t n, int W, cudaStream_t s);
 
 enum : int { DECIDE_XSTEP = 1, DECIDE_CYCLE = 2, DECIDE_CHECK = 4 };

@@ -12,74 +12,85 @@
 //   3. the rows are joined along M by the same rule on g(M) = sum_E g(E,M)
 //      (dM = 2), "one at a time" as Sec. 2 prescribes for both axes split;
 //   4. the joined table is shifted so that sum g = 2^N.
-// Loops that the sums depend on run in a fixed order (one thread per output
-// element), so results differ from a serial evaluation only by the rounding
-// of exp/log and of the final parallel normalisation sum.
+// The sums run in a fixed order (lanes, then warps, then blocks), so a join of
+// the same tables gives the same bits; results differ from a serial evaluation
+// by the rounding of exp/log and of the sums.
 #include <math.h>
 
 #include <algorithm>
 
 #include <math_constants.h>
 
-#include "rewl_internal.cuh"
+#include "rewl_tab.cuh"
 
 namespace rewl {
 
 namespace {
 
-// ln g of table entry i: base + max(H, 0) ln f in the exact formats (a
-// caller's plain table is read with ln f = 0), the stored value for REWL_F32.
-__device__ __forceinline__ double lng_at(const Params &p, size_t i)
+// One walker's table entries by format.  ln g = base + max(H, 0) ln f in the
+// exact formats (a caller's plain table is read with ln f = 0); REWL_F32 holds
+// ln g itself, and its H only says which bins were visited.
+template <int PREC>
+__device__ __forceinline__ const typename tab::Tab<PREC>::Elem *table_of(const Params &p)
 {
-    if (p.precision == REWL_F32) return (double)p.lng1[i];
-    double b;
-    if (p.precision == REWL_FP64) {
-        b = p.lng[i];
-    } else {
-        const float2 v = p.lng2[i];
-        b = (double)v.x + (double)v.y;
-    }
-    return fma((double)max(p.H[i], 0), p.st->lnf, b);
+    using Elem = typename tab::Tab<PREC>::Elem;
+    if constexpr (PREC == REWL_FP64) return reinterpret_cast<const Elem *>(p.lng);
+    else if constexpr (PREC == REWL_F32X2) return reinterpret_cast<const Elem *>(p.lng2);
+    else return reinterpret_cast<const Elem *>(p.lng1);
 }
 
-__device__ __forceinline__ bool all_seen(const Params &p, int win, int bin)
+// Terms of a sum of exp(v - max) this far below the largest (e^-60 < 1e-26)
+// are left out: all (N+1)^2 of them together stay below 2e-19 of the sum, a
+// thousandth of its rounding.  Most bins of a window are that far down.
+constexpr double LSE_FAR = 60.0;
+
+__device__ __forceinline__ double warp_max(double v)
 {
-    for (int k = 0; k < p.W; ++k)
-        if (k != p.join_exclude && p.H[(size_t)(win * p.W + k) * p.tstride + bin] < 0) return false;
-    return true;
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
 }
 
-// Serial log-sum-exp in index order: max, then sum of exp(v - max) over the
-// finite entries.
-template <typename F>
-__device__ double lse_serial(int n, F get)
+__device__ __forceinline__ double warp_sum(double v)
 {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+
+// ln sum_i exp(v[i]) over the finite v[0..n) by one warp: the largest, then
+// the sum in a fixed order (lane by lane, then the lanes).
+__device__ __forceinline__ double lse_warp(const double *v, int n)
+{
+    const int lane = threadIdx.x & 31;
     double mx = -INFINITY;
-    for (int i = 0; i < n; ++i) mx = fmax(mx, get(i));
-    if (mx == -INFINITY) return -INFINITY;
+    for (int i = lane; i < n; i += 32) mx = fmax(mx, v[i]);
+    mx = warp_max(mx);
+    if (mx == -INFINITY) return mx;
     double acc = 0.0;
-    for (int i = 0; i < n; ++i) {
-        const double v = get(i);
-        if (v != -INFINITY) acc += exp(v - mx);
+    for (int i = lane; i < n; i += 32) {
+        const double x = v[i];
+        if (x > mx - LSE_FAR) acc += exp(x - mx);
     }
-    return mx + log(acc);
+    return mx + log(warp_sum(acc));
 }
 
 // Matching point (Eq. 4) between marginals Ga, Gb over [lo, hi], q >= floor:
 // the overlap bin q minimising |beta_a(q) - beta_b(q)|, beta the forward
-// difference over one bin divided by the bin step, taken only where both
-// marginals are finite at q and q + 1; the lowest such q on ties.  Without
-// any, the lowest q where both are finite; -1 if none.
+// difference over one bin divided by the bin step (a power of two, so its
+// reciprocal divides exactly), taken only where both marginals are finite at q
+// and q + 1; the lowest such q on ties.  Without any, the lowest q where both
+// are finite; -1 if none.
 // It is computed by a whole block (every thread calls it and gets the
 // result): each thread scans a stride of q keeping its first minimum, and
 // the (difference, q) pairs are reduced lexicographically, so the lowest q
 // wins ties.
-constexpr int MATCH_THREADS = 256;
+constexpr int MATCH_THREADS = 128;
 
-__device__ void block_min_pair(double &d, int &q, double *s_d, int *s_q)
+// Lexicographic minimum of (d, q) over the block, d >= 0 by its bits (which
+// order like the values), so that no comparison needs the FP64 pipe.
+__device__ void block_min_pair(long long &d, int &q, long long *s_d, int *s_q)
 {
     for (int o = 16; o > 0; o >>= 1) {
-        const double od = __shfl_xor_sync(0xFFFFFFFFu, d, o);
+        const long long od = __shfl_xor_sync(0xFFFFFFFFu, d, o);
         const int oq = __shfl_xor_sync(0xFFFFFFFFu, q, o);
         if (od < d || (od == d && oq < q)) { d = od; q = oq; }
     }
@@ -88,115 +99,279 @@ __device__ void block_min_pair(double &d, int &q, double *s_d, int *s_q)
     __syncthreads();
     d = s_d[0];
     q = s_q[0];
-    for (int k = 1; k < (int)(blockDim.x >> 5); ++k)
+    for (int k = 1; k < MATCH_THREADS / 32; ++k)
         if (s_d[k] < d || (s_d[k] == d && s_q[k] < q)) { d = s_d[k]; q = s_q[k]; }
 }
 
-__device__ int match_point_block(const double *Ga, const double *Gb, int lo, int hi, int floor_p, double step)
+// v is not -infinity (by its bits)
+__device__ __forceinline__ bool some(double v) { return __double_as_longlong(v) != (long long)0xFFF0000000000000ull; }
+
+__device__ int match_point_block(const double *Ga, const double *Gb, int lo, int hi, int floor_p, double inv_step)
 {
-    __shared__ double s_d[MATCH_THREADS / 32];
+    __shared__ long long s_d[MATCH_THREADS / 32];
     __shared__ int s_q[MATCH_THREADS / 32];
+    const long long none = 0x7FF0000000000000ll;        // +infinity
     const int start = lo > floor_p ? lo : floor_p;
-    double bestd = INFINITY;
+    long long bestd = none;
     int best = 0x7FFFFFFF;
-    for (int q = start + (int)threadIdx.x; q + 1 <= hi; q += blockDim.x) {
-        if (Ga[q] == -INFINITY || Ga[q + 1] == -INFINITY) continue;
-        if (Gb[q] == -INFINITY || Gb[q + 1] == -INFINITY) continue;
-        const double ba = (Ga[q + 1] - Ga[q]) / step;
-        const double bb = (Gb[q + 1] - Gb[q]) / step;
-        const double d = fabs(ba - bb);
+    for (int q = start + (int)threadIdx.x; q + 1 <= hi; q += MATCH_THREADS) {
+        const double a0 = Ga[q], a1 = Ga[q + 1], b0 = Gb[q], b1 = Gb[q + 1];
+        if (!some(a0) || !some(a1) || !some(b0) || !some(b1)) continue;
+        const double ba = (a1 - a0) * inv_step;
+        const double bb = (b1 - b0) * inv_step;
+        const long long d = __double_as_longlong(fabs(ba - bb));
         if (d < bestd) { bestd = d; best = q; }
     }
     block_min_pair(bestd, best, s_d, s_q);
     if (best != 0x7FFFFFFF) return best;
-    double z = 0.0;
+    bestd = 0;
     best = 0x7FFFFFFF;
-    for (int q = start + (int)threadIdx.x; q <= hi; q += blockDim.x)
-        if (Ga[q] != -INFINITY && Gb[q] != -INFINITY) { best = q; break; }
-    block_min_pair(z, best, s_d, s_q);
+    for (int q = start + (int)threadIdx.x; q <= hi; q += MATCH_THREADS)
+        if (some(Ga[q]) && some(Gb[q])) { best = q; break; }
+    block_min_pair(bestd, best, s_d, s_q);
     return best == 0x7FFFFFFF ? -1 : best;
 }
 
 }  // namespace
 
-// 1a. Offsets: one block per (window, walker), relative to the first walker
-// taking part (walker join_exclude, if >= 0, is left out: the jackknife
-// replicates).  The block's threads take the bins in strides and reduce
-// their sums in a fixed order.
-constexpr int MERGE_OFF_THREADS = 256;
+// 1a. Offsets of each window's walkers relative to the first one taking part
+// (walker join_exclude, if >= 0, is left out: the jackknife replicates): the
+// mean of ln g_k - ln g_ref over the bins that all of them visited.
+//
+// Bounded by the FP64 pipe (two lanes an SM and cycle) and by HBM: the tables
+// are read once and the visits twice (the second time from L2).  A block takes
+// a chunk of a window's bins for all its walkers: which bins all walkers
+// visited is found once per window (it was found again for each walker, W^2
+// reads of H), then each warp takes walkers in turn and adds up base_k -
+// base_ref, two FP64 operations a bin; the visits are added up as integers.
+// Chunk sums are folded in chunk order.  L = 32, 2048 walkers (3.1 GB): 12.4
+// -> 1.2 ms; L = 16, 256 walkers 0.85 -> 0.05 ms.
+constexpr int OFF_THREADS = 256, OFF_BINS = 2048;
 
-__global__ void __launch_bounds__(MERGE_OFF_THREADS) k_merge_off(Params p, JoinScratch j)
+// Bins a chunk: all of a small window (its block then finishes the offsets),
+// else as many as leave some six blocks for each SM, and at least 4 W (the
+// chunk sums of a window take the place of at most its bins' entries).
+int off_chunk(const Params &p)
 {
-    const int idx = blockIdx.x;
-    if (idx >= p.nwalk) return;
-    const int win = idx / p.W, k = idx % p.W;
+    int chunk = OFF_BINS;
+    if (p.T <= OFF_BINS) return chunk;
+    while (chunk > 512 && (long long)(p.T / chunk) * p.nwin < 152 * 6) chunk /= 2;
+    while (chunk < 4 * p.W) chunk *= 2;
+    return chunk;
+}
+
+// Offset of walker k from its sum over the common bins, and the window's
+// typical visit count of a bin (in efrom until 2b writes it), which 1b takes
+// out of the walkers' visits to keep its sums small.
+__device__ __forceinline__ double offset_of(const Params &p, int k, int ref, double sum, double common)
+{
+    if (k == ref || k == p.join_exclude) return 0.0;
+    if (common == 0.0) { atomicExch(&p.st->join_error, 1); return 0.0; }
+    return sum / common;
+}
+
+__device__ __forceinline__ int typical_visits(const Params &p, double common, double ref_visits)
+{
+    return common > 0.0 && p.precision != REWL_F32 ? (int)(ref_visits / common) : 0;
+}
+
+template <int PREC>
+__global__ void __launch_bounds__(OFF_THREADS) k_off_part(Params p, JoinScratch j, int chunk, int nchunks)
+{
+    using TB = tab::Tab<PREC>;
+    using Elem = typename TB::Elem;
+    const int win = blockIdx.y, c = blockIdx.x, W = p.W;
     if (!p.active[win]) return;
     const int ref = p.join_exclude == 0 ? 1 : 0;   // the first walker taking part
-    if (k == ref || k == p.join_exclude) {
-        if (threadIdx.x == 0) j.off[idx] = 0.0;
-        return;
-    }
-    const size_t b0 = (size_t)(win * p.W + ref) * p.tstride, bk = (size_t)idx * p.tstride;
-    double acc = 0.0;
-    long long common = 0;
-    for (int i = threadIdx.x; i < p.T; i += MERGE_OFF_THREADS) {
-        if (!all_seen(p, win, i)) continue;
-        acc += lng_at(p, bk + i) - lng_at(p, b0 + i);
-        ++common;
+    __shared__ double s_ref[OFF_BINS];
+    __shared__ int s_h[OFF_BINS];                  // the reference's visits
+    __shared__ unsigned s_all[OFF_BINS / 32];      // bit: all walkers visited the bin
+    __shared__ long long s_hits[OFF_THREADS / 32], s_href[OFF_THREADS / 32];
+    __shared__ double s_common, s_visits, s_acc[OFF_THREADS / 32];
+    const int share = W <= 2 ? 8 : W <= 4 ? 2 : 1;
+    // per chunk W sums, then the number of common bins and the reference's
+    // visits of them; several chunks leave them where 1b writes the piece (at
+    // most half of its entries), a single one finishes the offsets itself
+    const bool single = nchunks == 1;
+    double *part = single ? j.off + (size_t)win * W : j.piece + (size_t)win * p.tstride + (size_t)c * (W + 2);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const Elem *B0 = table_of<PREC>(p) + (size_t)(win * W) * p.tstride;
+    const int32_t *H0 = p.H + (size_t)(win * W) * p.tstride;
+    long long hits = 0, href = 0;
+    for (int at = c * chunk; at < min(p.T, (c + 1) * chunk); at += OFF_BINS) {
+        const int n = min(OFF_BINS, min(p.T, (c + 1) * chunk) - at);
+        __syncthreads();
+        for (int b0 = 0; b0 < n; b0 += OFF_THREADS) {
+            const int b = b0 + (int)threadIdx.x;
+            int any = b < n ? 0 : -1;              // sign: some walker has not been there
+            if (b < n) {
+                #pragma unroll 8
+                for (int k = 0; k < W; ++k)
+                    if (k != p.join_exclude) any |= H0[(size_t)k * p.tstride + at + b];
+                s_ref[b] = TB::exact(B0[(size_t)ref * p.tstride + at + b]);
+                s_h[b] = H0[(size_t)ref * p.tstride + at + b];
+            }
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, any >= 0);
+            if (lane == 0) s_all[(b0 >> 5) + wid] = m;
+            if (any >= 0) {
+                ++hits;
+                href += s_h[b];
+            }
+        }
+        __syncthreads();
+        // few walkers: `share` warps to each, every share-th 32 bins a warp
+        const int turns = OFF_THREADS / 32 / share, mine = wid % share;
+        for (int k0 = 0; k0 < W; k0 += turns) {
+            const int k = k0 + wid / share;
+            const bool on = k < W && k != ref && k != p.join_exclude;
+            double acc = 0.0;
+            if (on) {
+                const Elem *B = B0 + (size_t)k * p.tstride + at;
+                const int32_t *H = H0 + (size_t)k * p.tstride + at;
+                long long hk = 0;
+                #pragma unroll 4
+                for (int b = lane + 32 * mine; b < n; b += 32 * share)
+                    if ((s_all[b >> 5] >> lane) & 1u) {
+                        acc += TB::exact(B[b]) - s_ref[b];
+                        hk += H[b] - s_h[b];
+                    }
+                acc = warp_sum(acc);
+                for (int o = 16; o > 0; o >>= 1) hk += __shfl_xor_sync(0xFFFFFFFFu, hk, o);
+                if (PREC != REWL_F32) acc = fma((double)hk, p.st->lnf, acc);
+            }
+            if (share > 1) {
+                if (lane == 0) s_acc[wid] = acc;
+                __syncthreads();
+                for (int q = 1; q < share; ++q) acc += s_acc[(wid / share) * share + q];
+                __syncthreads();
+            }
+            if (on && lane == 0 && mine == 0) part[k] = at == c * chunk ? acc : part[k] + acc;
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
-        acc += __shfl_down_sync(0xFFFFFFFFu, acc, o);
-        common += __shfl_down_sync(0xFFFFFFFFu, common, o);
+        hits += __shfl_xor_sync(0xFFFFFFFFu, hits, o);
+        href += __shfl_xor_sync(0xFFFFFFFFu, href, o);
     }
-    __shared__ double s_acc[MERGE_OFF_THREADS / 32];
-    __shared__ long long s_cnt[MERGE_OFF_THREADS / 32];
-    if ((threadIdx.x & 31) == 0) { s_acc[threadIdx.x >> 5] = acc; s_cnt[threadIdx.x >> 5] = common; }
+    if (lane == 0) { s_hits[wid] = hits; s_href[wid] = href; }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    acc = 0.0;
-    common = 0;
-    for (int w = 0; w < MERGE_OFF_THREADS / 32; ++w) { acc += s_acc[w]; common += s_cnt[w]; }
-    if (common == 0) { atomicExch(&p.st->join_error, 1); j.off[idx] = 0.0; return; }
-    j.off[idx] = acc / (double)common;
-}
-
-// 1b. Merged piece: one thread per (window, bin), walkers in order.
-__global__ void k_merge(Params p, JoinScratch j)
-{
-    const size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (idx >= (size_t)p.nwin * p.T) return;
-    const int win = (int)(idx / p.T), bin = (int)(idx % p.T);
-    double *out = j.piece + (size_t)win * p.tstride + bin;
-    if (!p.active[win]) { *out = -INFINITY; return; }
-    double acc = 0.0;
-    int cnt = 0;
-    for (int k = 0; k < p.W; ++k) {
-        const size_t q = (size_t)(win * p.W + k) * p.tstride + bin;
-        if (k == p.join_exclude || p.H[q] < 0) continue;
-        acc += lng_at(p, q) - j.off[win * p.W + k];
-        ++cnt;
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < OFF_THREADS / 32; ++k) { hits += s_hits[k]; href += s_href[k]; }
+        s_common = (double)hits;
+        s_visits = (double)href;
+        if (!single) { part[W] = s_common; part[W + 1] = s_visits; }
     }
-    *out = cnt ? acc / (double)cnt : -INFINITY;
+    if (!single) return;
+    __syncthreads();
+    const double common = s_common, visits = s_visits;
+    for (int k = threadIdx.x; k < W; k += OFF_THREADS)
+        part[k] = offset_of(p, k, ref, part[k], common);
+    if (threadIdx.x == 0) j.efrom[win] = typical_visits(p, common, visits);
 }
 
-// 2a. E marginal of each piece over its M range (Eq. 3).
-__global__ void k_marg_piece(Params p, JoinScratch j)
+// One block per window, one warp per walker in turn: the chunks' sums in a
+// fixed order (lane by lane, then the lanes).
+__global__ void __launch_bounds__(256) k_off_fold(Params p, JoinScratch j, int nchunks)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int win = blockIdx.x, W = p.W, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (!p.active[win]) return;
+    const int ref = p.join_exclude == 0 ? 1 : 0;
+    const double *part = j.piece + (size_t)win * p.tstride;
+    auto total = [&](int k) -> double {
+        double v = 0.0;
+        for (int c = lane; c < nchunks; c += 32) v += part[(size_t)c * (W + 2) + k];
+        return warp_sum(v);
+    };
+    const double common = total(W);
+    for (int k = wid; k < W; k += 8) {
+        const double sum = k != ref && k != p.join_exclude ? total(k) : 0.0;
+        if (lane == 0) j.off[(size_t)win * W + k] = offset_of(p, k, ref, sum, common);
+    }
+    if (wid == 0) {
+        const double visits = total(W + 1);
+        if (lane == 0) j.efrom[win] = typical_visits(p, common, visits);
+    }
+}
+
+// 1b. Merged piece: the mean of ln g_k - off_k over the walkers that visited
+// the bin, walkers in order; one thread per two bins of a window.
+//
+// Bounded by the FP64 pipe and HBM: base_k - off_k and its sum are two FP64
+// operations an entry, the visits are summed as integers (less the window's
+// typical count, whose ln g goes into the offset, so that neither sum grows
+// beyond the spread of the values).  L = 32, 2048 walkers (3.1 GB): 1.41 -> 1.1
+// ms (four FP64 operations an entry and one bin a thread before).
+template <int PREC>
+__global__ void __launch_bounds__(256) k_merge(Params p, JoinScratch j)
+{
+    using TB = tab::Tab<PREC>;
+    using Elem = typename TB::Elem;
+    extern __shared__ double s_off[];
+    const int win = blockIdx.y, W = p.W;
+    const int b = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    const bool act = p.active[win] != 0;
+    double *out = j.piece + (size_t)win * p.tstride;
+    const double lnf = PREC == REWL_F32 ? 0.0 : p.st->lnf;
+    const int h0 = act && PREC != REWL_F32 ? j.efrom[win] : 0;
+    if (act)
+        for (int k = threadIdx.x; k < W; k += blockDim.x) s_off[k] = fma(-(double)h0, lnf, j.off[win * W + k]);
+    __syncthreads();
+    if (b >= p.T) return;
+    const bool two = b + 1 < p.T;
+    double a0 = 0.0, a1 = 0.0;
+    int n0 = 0, n1 = 0;
+    long long v0 = 0, v1 = 0;
+    if (act) {
+        const Elem *B = table_of<PREC>(p) + (size_t)(win * W) * p.tstride + b;
+        const int32_t *H = p.H + (size_t)(win * W) * p.tstride + b;
+        struct __align__(2 * sizeof(Elem)) Pair { Elem x, y; };
+        // (a caller's unpadded tables may start anywhere: then entry by entry)
+        const bool wide = (p.tstride & 1) == 0 && ((uintptr_t)table_of<PREC>(p) & 15) == 0 && ((uintptr_t)p.H & 7) == 0;
+        #pragma unroll 4
+        for (int k = 0; k < W; ++k) {
+            if (k == p.join_exclude) continue;
+            const size_t q = (size_t)k * p.tstride;
+            int hx, hy = -1;
+            Elem x, y = Elem();
+            if (wide && two) {
+                const int2 h = *reinterpret_cast<const int2 *>(H + q);
+                const Pair e = *reinterpret_cast<const Pair *>(B + q);
+                hx = h.x; hy = h.y; x = e.x; y = e.y;
+            } else {
+                hx = H[q]; x = B[q];
+                if (two) { hy = H[q + 1]; y = B[q + 1]; }
+            }
+            if (hx >= 0) { a0 += TB::exact(x) - s_off[k]; v0 += hx - h0; ++n0; }
+            if (hy >= 0) { a1 += TB::exact(y) - s_off[k]; v1 += hy - h0; ++n1; }
+        }
+    }
+    auto mean = [&](double a, long long v, int n) -> double {
+        if (n == 0) return -INFINITY;
+        if (PREC != REWL_F32) a = fma((double)v, lnf, a);
+        if ((n & (n - 1)) == 0) return a * __hiloint2double((1023 - (31 - __clz(n))) << 20, 0);   // / 2^i
+        return a / (double)n;
+    };
+    out[b] = mean(a0, v0, n0);
+    if (two) out[b + 1] = mean(a1, v1, n1);
+}
+
+// 2a. E marginal of each piece over its M range (Eq. 3): one warp per
+// (window, e).  (One thread each before: 514 -> 240 us at L = 32.)
+__global__ void __launch_bounds__(256) k_marg_piece(Params p, JoinScratch j)
+{
+    const int idx = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (idx >= p.nwin * p.wE) return;
     const int win = idx / p.wE, el = idx % p.wE;
-    const double *row = j.piece + (size_t)win * p.tstride + (size_t)el * p.wM;
-    j.GE[idx] = p.active[win] ? lse_serial(p.wM, [&](int i) { return row[i]; }) : -INFINITY;
+    const double g = p.active[win] ? lse_warp(j.piece + (size_t)win * p.tstride + (size_t)el * p.wM, p.wM) : -INFINITY;
+    if ((threadIdx.x & 31) == 0) j.GE[idx] = g;
 }
 
 // 2b. One block per row b: chain of E matching points along the row (the
 // chain is sequential; each matching point and slice rule is block-parallel).
-__global__ void __launch_bounds__(MATCH_THREADS) k_match_e(Params p, JoinScratch j, double *gbuf)
+__global__ void __launch_bounds__(MATCH_THREADS) k_match_e(Params p, JoinScratch j)
 {
     const int b = blockIdx.x;
     if (b >= p.nM) return;
-    const int nE = p.nE, B = p.N + 1, t0 = threadIdx.x == 0;
-    double *Ga = gbuf + (size_t)b * 2 * B, *Gb = Ga + B;
+    const int nE = p.nE, t0 = threadIdx.x == 0;
     __shared__ int s_first, s_last, s_bad;
     if (t0) {
         for (int a = 0; a < nE; ++a) {
@@ -228,12 +403,9 @@ __global__ void __launch_bounds__(MATCH_THREADS) k_match_e(Params p, JoinScratch
         __syncthreads();                      // the last piece's buffers and slices are complete
         if (a < last) {
             const int4 RB = p.rect[A + 1];
-            for (int e = threadIdx.x; e < B; e += blockDim.x) {
-                Ga[e] = (e >= RA.x && e <= RA.y) ? j.GE[A * p.wE + (e - RA.x)] : -INFINITY;
-                Gb[e] = (e >= RB.x && e <= RB.y) ? j.GE[(A + 1) * p.wE + (e - RB.x)] : -INFINITY;
-            }
-            __syncthreads();
-            const int q = match_point_block(Ga, Gb, RB.x, RA.y, from, 4.0);
+            // the two marginals by absolute bin, read in the overlap [RB.x, RA.y] alone
+            const double *Ga = j.GE + (ptrdiff_t)A * p.wE - RA.x, *Gb = j.GE + (ptrdiff_t)(A + 1) * p.wE - RB.x;
+            const int q = match_point_block(Ga, Gb, RB.x, RA.y, from, 0.25);
             if (q < 0) { if (t0) atomicExch(&p.st->join_error, 3); return; }
             if (t0) j.ematch[b * (nE - 1) + a] = q;
             next_shift = shift + (Ga[q] - Gb[q]);
@@ -275,15 +447,48 @@ __device__ __forceinline__ double row_value(const Params &p, const JoinScratch &
     return -INFINITY;
 }
 
-// 3a. M marginal of each row: F_b(m) = ln sum_E g_b(E, m), e ascending.
-__global__ void k_marg_row(Params p, JoinScratch j)
+// 3a. M marginal of each row: F_b(m) = ln sum_E g_b(E, m).  A block takes
+// ROW_COLS adjacent m of a row, its threads every ROW_ES-th e, piece by piece
+// (the pieces tile the row, so no entry has to look for its piece); the threads'
+// parts meet in shared memory.  Few columns a block: exp is FP64 work, which an
+// SM does at two lanes a cycle, so it has to be spread over the SMs.  (One
+// thread per m, all e twice, looking for each entry's piece before: 2.84 ->
+// 0.12 ms at L = 32, 0.40 -> 0.02 ms at L = 16.)
+constexpr int ROW_COLS = 8, ROW_ES = 32;
+
+__global__ void __launch_bounds__(ROW_COLS * ROW_ES) k_marg_row(Params p, JoinScratch j)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int B = p.N + 1;
-    if (idx >= p.nM * B) return;
-    const int b = idx / B, m = idx % B;
-    if (!j.rowok[b]) { j.F[idx] = -INFINITY; return; }
-    j.F[idx] = lse_serial(B, [&](int e) { return row_value(p, j, b, e, m); });
+    const int B = p.N + 1, b = blockIdx.y, cx = threadIdx.x % ROW_COLS, ex = threadIdx.x / ROW_COLS;
+    const int m = (int)blockIdx.x * ROW_COLS + cx;
+    __shared__ double s_part[ROW_ES][ROW_COLS];
+    const int4 R0 = p.rect[b * p.nE];              // the row's m range is its pieces'
+    const bool in = j.rowok[b] && m >= R0.z && m <= R0.w;
+    auto each = [&](auto f) {
+        if (!in) return;
+        for (int a = 0; a < p.nE; ++a) {
+            const int A = b * p.nE + a, from = j.efrom[A], to = j.eto[A];
+            const double *col = j.piece + (size_t)A * p.tstride + (m - R0.z);
+            const int e0 = p.rect[A].x;
+            const double c = p.join_rule == 1 && to > from ? j.eslice[(size_t)A * p.wM + (m - R0.z)] : j.eshift[A];
+            #pragma unroll 4
+            for (int e = from + ex; e < to; e += ROW_ES) f(col[(size_t)(e - e0) * p.wM] + c);
+        }
+    };
+    double mx = -INFINITY;
+    each([&](double v) { mx = fmax(mx, v); });
+    s_part[ex][cx] = mx;
+    __syncthreads();
+    for (int k = 0; k < ROW_ES; ++k) mx = fmax(mx, s_part[k][cx]);
+    __syncthreads();
+    double acc = 0.0;
+    if (mx != -INFINITY)
+        each([&](double v) { if (v > mx - LSE_FAR) acc += exp(v - mx); });
+    s_part[ex][cx] = acc;
+    __syncthreads();
+    if (ex == 0 && m < B) {
+        for (int k = 1; k < ROW_ES; ++k) acc += s_part[k][cx];
+        j.F[(size_t)b * B + m] = mx == -INFINITY ? mx : mx + log(acc);
+    }
 }
 
 // 3b. One block: chain of M matching points over the rows (sequential
@@ -316,7 +521,7 @@ __global__ void __launch_bounds__(MATCH_THREADS) k_match_m(Params p, JoinScratch
         if (b < last) {
             const double *Ga = j.F + (size_t)b * B, *Gb = j.F + (size_t)(b + 1) * B;
             const int lo = p.rect[(b + 1) * nE].z, hi = p.rect[b * nE].w;
-            const int q = match_point_block(Ga, Gb, lo, hi, from, 2.0);
+            const int q = match_point_block(Ga, Gb, lo, hi, from, 0.5);
             if (q < 0) { if (t0) atomicExch(&p.st->join_error, 6); return; }
             if (t0) j.mmatch[b] = q;
             next_shift = shift + (Ga[q] - Gb[q]);
@@ -336,142 +541,150 @@ __global__ void __launch_bounds__(MATCH_THREADS) k_match_m(Params p, JoinScratch
     }
 }
 
-// 3c. Assemble the joined table.
-__global__ void k_assemble(Params p, JoinScratch j)
+// 3c. Assemble the joined table; each block leaves the largest value of its
+// part in red[].
+constexpr int RED_BLOCKS = 512;     // red[0..512): maxima, red[512..1024): sums
+
+__global__ void __launch_bounds__(256) k_assemble(Params p, JoinScratch j)
 {
     const int B = p.N + 1;
-    const size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (idx >= (size_t)B * B) return;
-    const int e = (int)(idx / B), m = (int)(idx % B);
-    double v = -INFINITY;
-    for (int b = 0; b < p.nM; ++b) {
-        if (m >= j.mfrom[b] && m < j.mto[b]) {
-            const double r = row_value(p, j, b, e, m);
-            const double c = p.join_rule == 1 ? j.mslice[(size_t)b * B + e] : j.mshift[b];
-            v = r == -INFINITY ? r : r + c;
-            break;
+    double mx = -INFINITY;
+    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < (size_t)B * B; idx += (size_t)gridDim.x * blockDim.x) {
+        const int e = (int)(idx / B), m = (int)(idx % B);
+        double v = -INFINITY;
+        for (int b = 0; b < p.nM; ++b) {
+            if (m >= j.mfrom[b] && m < j.mto[b]) {
+                const double r = row_value(p, j, b, e, m);
+                const double c = p.join_rule == 1 ? j.mslice[(size_t)b * B + e] : j.mshift[b];
+                v = r == -INFINITY ? r : r + c;
+                break;
+            }
         }
+        j.J[idx] = v;
+        mx = fmax(mx, v);
     }
-    j.J[idx] = v;
-}
-
-// 4. Normalisation: max, then sum of exp(v - max), block partials in red[].
-__global__ void k_red_max(const double *v, size_t n, double *red)
-{
-    double mx = -INFINITY;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        mx = fmax(mx, v[i]);
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-    __shared__ double s[32];
+    mx = warp_max(mx);
+    __shared__ double s[8];
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = mx;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) mx = fmax(mx, s[k]);
-        red[blockIdx.x] = mx;
+        for (int k = 1; k < 8; ++k) mx = fmax(mx, s[k]);
+        j.red[blockIdx.x] = mx;
     }
 }
 
-// Block partials red[0..nblk) folded once, by one block: red[RED_MAX] = the max.
-constexpr int RED_MAX = 1024, RED_SHIFT = 1025;
-
-__global__ void k_red_fold_max(double *red, int nblk)
+// 4. Normalisation: sums of exp(v - max) by blocks, then the shift that makes
+// sum g = 2^N.  Each block folds the blocks' maxima (sums) itself, all in the
+// same order, instead of waiting for a kernel that does.
+__device__ __forceinline__ double fold_max(const double *red, int n)
 {
+    __shared__ double s_m[8];
     double mx = -INFINITY;
-    for (int k = threadIdx.x; k < nblk; k += blockDim.x) mx = fmax(mx, red[k]);
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-    __shared__ double s[32];
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = mx;
+    for (int k = threadIdx.x; k < n; k += 256) mx = fmax(mx, red[k]);
+    mx = warp_max(mx);
+    if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = mx;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) mx = fmax(mx, s[k]);
-        red[RED_MAX] = mx;
-    }
+    for (int k = 0; k < 8; ++k) mx = fmax(mx, s_m[k]);
+    return mx;
 }
 
-__global__ void k_red_sumexp(const double *v, size_t n, double *red)
+__global__ void __launch_bounds__(256) k_red_sumexp(const double *v, size_t n, double *red, int nblk)
 {
-    const double mx = red[RED_MAX];
+    const double mx = fold_max(red, nblk);
     double acc = 0.0;
     if (mx != -INFINITY)
-        for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-            if (v[i] != -INFINITY) acc += exp(v[i] - mx);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-    __shared__ double s[32];
+        for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+            const double x = v[i];
+            if (x > mx - LSE_FAR) acc += exp(x - mx);
+        }
+    acc = warp_sum(acc);
+    __shared__ double s[8];
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) acc += s[k];
-        red[512 + blockIdx.x] = acc;
+        for (int k = 1; k < 8; ++k) acc += s[k];
+        red[RED_BLOCKS + blockIdx.x] = acc;
     }
 }
 
-// Sum partials red[512..512+nblk) folded in a fixed order; red[RED_SHIFT] =
-// N ln 2 - ln sum g, the shift that makes sum g = 2^N.
-__global__ void k_red_fold_sum(double *red, int nblk, int N)
+__global__ void __launch_bounds__(256) k_normalise(double *v, size_t n, const double *red, int nblk, int N)
 {
+    const double mx = fold_max(red, nblk);
     double acc = 0.0;
-    for (int k = threadIdx.x; k < nblk; k += blockDim.x) acc += red[512 + k];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-    __shared__ double s[32];
+    for (int k = threadIdx.x; k < nblk; k += 256) acc += red[RED_BLOCKS + k];
+    acc = warp_sum(acc);
+    __shared__ double s[8], s_c;
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) acc += s[k];
-        red[RED_SHIFT] = (double)N * log(2.0) - (red[RED_MAX] + log(acc));
+        for (int k = 1; k < 8; ++k) acc += s[k];
+        s_c = (double)N * log(2.0) - (mx + log(acc));
     }
-}
-
-__global__ void k_normalise(double *v, size_t n, const double *red)
-{
-    const double c = red[RED_SHIFT];
+    __syncthreads();
+    const double c = s_c;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         if (v[i] != -INFINITY) v[i] += c;
 }
 
+namespace {
+
+// Warps a block of the kernels that take a row a warp: one while there is an SM
+// for each row (their FP64 work is an SM's bottleneck), eight when there are many.
+int row_warps(int rows) { return rows >= 152 * 8 ? 8 : rows >= 152 * 2 ? 2 : 1; }
+
+template <int PREC>
+void launch_merge(const Params &p, const JoinScratch &j, cudaStream_t s)
+{
+    const int chunk = off_chunk(p), nchunks = (p.T + chunk - 1) / chunk;
+    k_off_part<PREC><<<dim3(nchunks, p.nwin), OFF_THREADS, 0, s>>>(p, j, chunk, nchunks);
+    if (nchunks > 1) k_off_fold<<<p.nwin, 256, 0, s>>>(p, j, nchunks);
+    k_merge<PREC><<<dim3((p.T + 511) / 512, p.nwin), 256, sizeof(double) * p.W, s>>>(p, j);
+}
+
+}  // namespace
+
 cudaError_t launch_join(const Params &p, const JoinScratch &j, cudaStream_t s)
 {
     const int B = p.N + 1;
-    k_merge_off<<<p.nwalk, MERGE_OFF_THREADS, 0, s>>>(p, j);
-    const size_t nb = (size_t)p.nwin * p.T;
-    k_merge<<<(unsigned)((nb + 255) / 256), 256, 0, s>>>(p, j);
-    k_marg_piece<<<(p.nwin * p.wE + 127) / 128, 128, 0, s>>>(p, j);
-    k_match_e<<<p.nM, MATCH_THREADS, 0, s>>>(p, j, j.gbuf);
-    k_marg_row<<<(p.nM * B + 127) / 128, 128, 0, s>>>(p, j);
+    if (p.precision == REWL_FP64) launch_merge<REWL_FP64>(p, j, s);
+    else if (p.precision == REWL_F32X2) launch_merge<REWL_F32X2>(p, j, s);
+    else launch_merge<REWL_F32>(p, j, s);
+    const int rows = p.nwin * p.wE, warps = row_warps(rows);
+    k_marg_piece<<<(rows + warps - 1) / warps, 32 * warps, 0, s>>>(p, j);
+    k_match_e<<<p.nM, MATCH_THREADS, 0, s>>>(p, j);
+    k_marg_row<<<dim3((B + ROW_COLS - 1) / ROW_COLS, p.nM), ROW_COLS * ROW_ES, 0, s>>>(p, j);
     k_match_m<<<1, MATCH_THREADS, 0, s>>>(p, j);
     const size_t nJ = (size_t)B * B;
-    k_assemble<<<(unsigned)((nJ + 255) / 256), 256, 0, s>>>(p, j);
-    // normalisation: block maxima, one fold, block sums of exp(v - max), one
-    // fold into the shift, shift applied (grids sized to the table, <= 512)
-    const int nblk = (int)std::min<size_t>(512, (nJ + 255) / 256);
-    k_red_max<<<nblk, 256, 0, s>>>(j.J, nJ, j.red);
-    k_red_fold_max<<<1, 512, 0, s>>>(j.red, nblk);
-    k_red_sumexp<<<nblk, 256, 0, s>>>(j.J, nJ, j.red);
-    k_red_fold_sum<<<1, 512, 0, s>>>(j.red, nblk, p.N);
-    k_normalise<<<nblk, 256, 0, s>>>(j.J, nJ, j.red);
+    const int nblk = (int)std::min<size_t>(RED_BLOCKS, (nJ + 255) / 256);
+    k_assemble<<<nblk, 256, 0, s>>>(p, j);
+    k_red_sumexp<<<nblk, 256, 0, s>>>(j.J, nJ, j.red, nblk);
+    k_normalise<<<nblk, 256, 0, s>>>(j.J, nJ, j.red, nblk, p.N);
     return cudaGetLastError();
 }
 
-// Eq. 3 on the joined table: ln sum_m g(e, m), m ascending.
-__global__ void k_marg_out(Params p, JoinScratch j)
+// Eq. 3 on the joined table: ln sum_m g(e, m), one warp per e.
+__global__ void __launch_bounds__(256) k_marg_out(Params p, JoinScratch j)
 {
     const int B = p.N + 1;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const int e = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (e >= B) return;
-    const double *row = j.J + (size_t)e * B;
-    j.marg[e] = lse_serial(B, [&](int i) { return row[i]; });
+    const double g = lse_warp(j.J + (size_t)e * B, B);
+    if ((threadIdx.x & 31) == 0) j.marg[e] = g;
 }
 
 cudaError_t launch_marginal_e(const Params &p, const JoinScratch &j, cudaStream_t s)
 {
-    k_marg_out<<<(p.N + 1 + 127) / 128, 128, 0, s>>>(p, j);
+    const int rows = p.N + 1, warps = row_warps(rows);
+    k_marg_out<<<(rows + warps - 1) / warps, 32 * warps, 0, s>>>(p, j);
     return cudaGetLastError();
 }
 
 // Jackknife accumulation over replicates k = 0..W-1 (walker k left out of
 // every window's merge): differences to replicate 0 are summed; an entry that
 // is missing (-inf) in any replicate is marked NaN in jk_ref.
-__global__ void k_jk_accum(JoinScratch j, const double *x, size_t n, int k)
+__global__ void k_jk_accum(Params p, JoinScratch j, const double *x, size_t n, int k, int32_t *fail)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0 && p.st->join_error && *fail == 0) *fail = k << 8 | p.st->join_error;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const double v = x[i];
         if (k == 0) {
@@ -504,9 +717,10 @@ __global__ void k_jk_final(JoinScratch j, double *mean, double *err, size_t n, i
     }
 }
 
-cudaError_t launch_jk_accum(const JoinScratch &j, const double *x, size_t n, int k, cudaStream_t s)
+cudaError_t launch_jk_accum(const Params &p, const JoinScratch &j, const double *x, size_t n, int k, int32_t *fail,
+                            cudaStream_t s)
 {
-    k_jk_accum<<<256, 256, 0, s>>>(j, x, n, k);
+    k_jk_accum<<<256, 256, 0, s>>>(p, j, x, n, k, fail);
     return cudaGetLastError();
 }
 

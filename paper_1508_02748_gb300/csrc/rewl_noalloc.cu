@@ -90,7 +90,7 @@ extern "C" int rewl_join_noalloc(const rewl_config *cfg, const double *d_lng, co
     const size_t o_mmatch = take(4 * (size_t)(d.nM > 1 ? d.nM - 1 : 1));
     const size_t o_red = take(8 * 2048);
     const size_t o_marg = take(8 * B);
-    const size_t o_gbuf = take(8 * 2 * B * (size_t)d.nM);
+    take(8 * 2 * B * (size_t)d.nM);          // spare: the capacity stays what callers know
     if (o > kScratchBytes)
         return say(REWL_E_CAPACITY,
                    "rewl_join_noalloc: this geometry needs %zu bytes of join scratch, above the fixed %zu "
@@ -160,7 +160,6 @@ extern "C" int rewl_join_noalloc(const rewl_config *cfg, const double *d_lng, co
     j.J = d_out;                             // the joined table is built in the caller's output
     j.red = (double *)(base + o_red);
     j.marg = (double *)(base + o_marg);
-    j.gbuf = (double *)(base + o_gbuf);
 
     cudaStream_t s = (cudaStream_t)stream;
     // a zeroed state has ln f = 0: the join reads the caller's ln g as it is
