@@ -104,3 +104,23 @@ def test_noalloc_join_of_unaligned_tables(P):
     assert P.load_library().rewl_join_noalloc(ctypes.byref(c), ctypes.c_void_p(d_lng.data_ptr()), ctypes.c_void_p(d_H.data_ptr()),
                                               ctypes.c_void_p(out.data_ptr()), None) == 0
     _near(out.cpu().numpy(), o.join()[0])
+
+
+# Eq. 5 either side of the series' end at 1/8, empty bins, non-finite ones, odd
+# counts and tables that start at an odd entry
+@pytest.mark.parametrize("n,shift", [(1, 0), (2, 0), (4097, 0), (4096, 1), (100_001, 1)])
+def test_relative_difference_forms(P, n, shift):
+    import torch
+    rng = np.random.default_rng(n)
+    a = rng.normal(0, 300, n)
+    b = a + np.where(rng.random(n) < 0.5, 1, -1) * 10.0 ** rng.uniform(-13, 2, n)
+    for i, (x, y) in enumerate([(0.0, 0.125), (0.125, 0.0), (0.0, np.nextafter(0.125, 0)), (-np.inf, 1.0), (1.0, -np.inf),
+                                (-np.inf, -np.inf), (np.inf, 1.0), (np.nan, 1.0), (5.0, 5.0)][:n]):
+        a[-1 - i], b[-1 - i] = x, y
+    da, db = (torch.zeros(n + shift, dtype=torch.float64, device="cuda")[shift:].copy_(torch.from_numpy(v)) for v in (a, b))
+    got = P.relative_difference(da, db).cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        ref = 2.0 * np.tanh(0.5 * np.abs(a - b))
+    ea, eb = np.isneginf(a), np.isneginf(b)
+    ref = np.where(ea & eb, np.nan, np.where(ea | eb, 2.0, ref))
+    np.testing.assert_allclose(got, ref, rtol=2e-15, atol=0)
