@@ -52,33 +52,46 @@ __device__ __forceinline__ bool pairs_aligned(const Params &p)
 // thousandth of its rounding.  Most bins of a window are that far down.
 constexpr double LSE_FAR = 60.0;
 
-__device__ __forceinline__ double warp_max(double v)
-{
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-    return v;
-}
-
 __device__ __forceinline__ double warp_sum(double v)
 {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
     return v;
 }
 
-// ln sum_i exp(v[i]) over the finite v[0..n) by one warp: the largest, then
-// the sum in a fixed order (lane by lane, then the lanes).
+// Sums of exp(v - top) compare values by their upper words, which order like
+// them (an FP64 comparison occupies its pipe like an addition does): the top
+// needs only to be near the largest value, and a term is left out where it is
+// certainly LSE_FAR below.
+__device__ __forceinline__ int order_of(double v)
+{
+    const int h = __double2hiint(v);
+    return h ^ ((h >> 31) & 0x7FFFFFFF);
+}
+
+constexpr int ORDER_NONE = (int)0xFFF00000 ^ 0x7FFFFFFF;       // of -infinity
+
+__device__ __forceinline__ double top_of(int order)
+{
+    return __hiloint2double(order ^ ((order >> 31) & 0x7FFFFFFF), 0);
+}
+
+// ln sum_i exp(v[i]) over the finite v[0..n) by one warp: the top, then the
+// sum in a fixed order (lane by lane, then the lanes).
 __device__ __forceinline__ double lse_warp(const double *v, int n)
 {
     const int lane = threadIdx.x & 31;
-    double mx = -INFINITY;
-    for (int i = lane; i < n; i += 32) mx = fmax(mx, v[i]);
-    mx = warp_max(mx);
-    if (mx == -INFINITY) return mx;
+    int mo = ORDER_NONE;
+    for (int i = lane; i < n; i += 32) mo = max(mo, order_of(v[i]));
+    mo = __reduce_max_sync(0xFFFFFFFFu, mo);
+    if (mo == ORDER_NONE) return -INFINITY;
+    const double top = top_of(mo);
+    const int far = order_of(top - LSE_FAR);
     double acc = 0.0;
     for (int i = lane; i < n; i += 32) {
         const double x = v[i];
-        if (x > mx - LSE_FAR) acc += exp(x - mx);
+        if (order_of(x) >= far) acc += exp(x - top);
     }
-    return mx + log(warp_sum(acc));
+    return top + log(warp_sum(acc));
 }
 
 // Matching point (Eq. 4) between marginals Ga, Gb over [lo, hi], q >= floor:
@@ -429,7 +442,7 @@ __global__ void __launch_bounds__(MATCH_THREADS) k_match_e(Params p, JoinScratch
                 double *sb = j.eslice + (size_t)(A + 1) * p.wM;
                 for (int ml = threadIdx.x; ml < p.wM; ml += blockDim.x) {
                     const double va = pa[ml], vb = pb[ml];
-                    sb[ml] = sa[ml] + ((va != -INFINITY && vb != -INFINITY) ? va - vb : Ga[q] - Gb[q]);
+                    sb[ml] = sa[ml] + (some(va) && some(vb) ? va - vb : Ga[q] - Gb[q]);
                 }
             }
             to = q;
@@ -452,7 +465,7 @@ __device__ __forceinline__ double row_value(const Params &p, const JoinScratch &
             if (m < R.z || m > R.w) return -INFINITY;
             const double v = j.piece[(size_t)A * p.tstride + (size_t)(e - R.x) * p.wM + (m - R.z)];
             const double c = p.join_rule == 1 ? j.eslice[(size_t)A * p.wM + (m - R.z)] : j.eshift[A];
-            return v == -INFINITY ? v : v + c;
+            return some(v) ? v + c : v;
         }
     }
     return -INFINITY;
@@ -485,20 +498,23 @@ __global__ void __launch_bounds__(ROW_COLS * ROW_ES) k_marg_row(Params p, JoinSc
             for (int e = from + ex; e < to; e += ROW_ES) f(col[(size_t)(e - e0) * p.wM] + c);
         }
     };
-    double mx = -INFINITY;
-    each([&](double v) { mx = fmax(mx, v); });
-    s_part[ex][cx] = mx;
+    __shared__ int s_top[ROW_ES][ROW_COLS];
+    int mo = ORDER_NONE;
+    each([&](double v) { mo = max(mo, order_of(v)); });
+    s_top[ex][cx] = mo;
     __syncthreads();
-    for (int k = 0; k < ROW_ES; ++k) mx = fmax(mx, s_part[k][cx]);
-    __syncthreads();
+    for (int k = 0; k < ROW_ES; ++k) mo = max(mo, s_top[k][cx]);
+    const double top = top_of(mo);
     double acc = 0.0;
-    if (mx != -INFINITY)
-        each([&](double v) { if (v > mx - LSE_FAR) acc += exp(v - mx); });
+    if (mo != ORDER_NONE) {
+        const int far = order_of(top - LSE_FAR);
+        each([&](double v) { if (order_of(v) >= far) acc += exp(v - top); });
+    }
     s_part[ex][cx] = acc;
     __syncthreads();
     if (ex == 0 && m < B) {
         for (int k = 1; k < ROW_ES; ++k) acc += s_part[k][cx];
-        j.F[(size_t)b * B + m] = mx == -INFINITY ? mx : mx + log(acc);
+        j.F[(size_t)b * B + m] = mo == ORDER_NONE ? -INFINITY : top + log(acc);
     }
 }
 
@@ -540,7 +556,7 @@ __global__ void __launch_bounds__(MATCH_THREADS) k_match_m(Params p, JoinScratch
                 for (int e = threadIdx.x; e < B; e += blockDim.x) {
                     const double va = row_value(p, j, b, e, q), vb = row_value(p, j, b + 1, e, q);
                     j.mslice[(size_t)(b + 1) * B + e] = j.mslice[(size_t)b * B + e]
-                        + ((va != -INFINITY && vb != -INFINITY) ? va - vb : Ga[q] - Gb[q]);
+                        + (some(va) && some(vb) ? va - vb : Ga[q] - Gb[q]);
                 }
             to = q;
         } else {
@@ -552,14 +568,14 @@ __global__ void __launch_bounds__(MATCH_THREADS) k_match_m(Params p, JoinScratch
     }
 }
 
-// 3c. Assemble the joined table; each block leaves the largest value of its
-// part in red[].
-constexpr int RED_BLOCKS = 512;     // red[0..512): maxima, red[512..1024): sums
+// 3c. Assemble the joined table; each block leaves the order of the largest
+// value of its part in red[].
+constexpr int RED_BLOCKS = 512;     // red[]: 512 maxima (their order), then from entry 512 on the sums
 
 __global__ void __launch_bounds__(256) k_assemble(Params p, JoinScratch j)
 {
     const int B = p.N + 1;
-    double mx = -INFINITY;
+    int mo = ORDER_NONE;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < (size_t)B * B; idx += (size_t)gridDim.x * blockDim.x) {
         const int e = (int)(idx / B), m = (int)(idx % B);
         double v = -INFINITY;
@@ -567,47 +583,50 @@ __global__ void __launch_bounds__(256) k_assemble(Params p, JoinScratch j)
             if (m >= j.mfrom[b] && m < j.mto[b]) {
                 const double r = row_value(p, j, b, e, m);
                 const double c = p.join_rule == 1 ? j.mslice[(size_t)b * B + e] : j.mshift[b];
-                v = r == -INFINITY ? r : r + c;
+                v = some(r) ? r + c : r;
                 break;
             }
         }
         j.J[idx] = v;
-        mx = fmax(mx, v);
+        mo = max(mo, order_of(v));
     }
-    mx = warp_max(mx);
-    __shared__ double s[8];
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = mx;
+    mo = __reduce_max_sync(0xFFFFFFFFu, mo);
+    __shared__ int s[8];
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = mo;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < 8; ++k) mx = fmax(mx, s[k]);
-        j.red[blockIdx.x] = mx;
+        for (int k = 1; k < 8; ++k) mo = max(mo, s[k]);
+        reinterpret_cast<int *>(j.red)[blockIdx.x] = mo;
     }
 }
 
 // 4. Normalisation: sums of exp(v - max) by blocks, then the shift that makes
 // sum g = 2^N.  Each block folds the blocks' maxima (sums) itself, all in the
 // same order, instead of waiting for a kernel that does.
-__device__ __forceinline__ double fold_max(const double *red, int n)
+__device__ __forceinline__ int fold_max(const double *red, int n)
 {
-    __shared__ double s_m[8];
-    double mx = -INFINITY;
-    for (int k = threadIdx.x; k < n; k += 256) mx = fmax(mx, red[k]);
-    mx = warp_max(mx);
-    if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = mx;
+    __shared__ int s_m[8];
+    int mo = ORDER_NONE;
+    for (int k = threadIdx.x; k < n; k += 256) mo = max(mo, reinterpret_cast<const int *>(red)[k]);
+    mo = __reduce_max_sync(0xFFFFFFFFu, mo);
+    if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = mo;
     __syncthreads();
-    for (int k = 0; k < 8; ++k) mx = fmax(mx, s_m[k]);
-    return mx;
+    for (int k = 0; k < 8; ++k) mo = max(mo, s_m[k]);
+    return mo;
 }
 
 __global__ void __launch_bounds__(256) k_red_sumexp(const double *v, size_t n, double *red, int nblk)
 {
-    const double mx = fold_max(red, nblk);
+    const int mo = fold_max(red, nblk);
+    const double top = top_of(mo);
     double acc = 0.0;
-    if (mx != -INFINITY)
+    if (mo != ORDER_NONE) {
+        const int far = order_of(top - LSE_FAR);
         for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
             const double x = v[i];
-            if (x > mx - LSE_FAR) acc += exp(x - mx);
+            if (order_of(x) >= far) acc += exp(x - top);
         }
+    }
     acc = warp_sum(acc);
     __shared__ double s[8];
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = acc;
@@ -620,7 +639,7 @@ __global__ void __launch_bounds__(256) k_red_sumexp(const double *v, size_t n, d
 
 __global__ void __launch_bounds__(256) k_normalise(double *v, size_t n, const double *red, int nblk, int N)
 {
-    const double mx = fold_max(red, nblk);
+    const double top = top_of(fold_max(red, nblk));
     double acc = 0.0;
     for (int k = threadIdx.x; k < nblk; k += 256) acc += red[RED_BLOCKS + k];
     acc = warp_sum(acc);
@@ -629,12 +648,14 @@ __global__ void __launch_bounds__(256) k_normalise(double *v, size_t n, const do
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int k = 1; k < 8; ++k) acc += s[k];
-        s_c = (double)N * log(2.0) - (mx + log(acc));
+        s_c = (double)N * log(2.0) - (top + log(acc));
     }
     __syncthreads();
     const double c = s_c;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        if (v[i] != -INFINITY) v[i] += c;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const double x = v[i];
+        if (some(x)) v[i] = x + c;
+    }
 }
 
 namespace {
