@@ -203,6 +203,7 @@ __device__ __forceinline__ int typical_visits(const Params &p, double common, do
 template <int PREC>
 __global__ void __launch_bounds__(OFF_THREADS) k_off_part(Params p, JoinScratch j, int chunk, int nchunks)
 {
+    after_previous();
     using TB = tab::Tab<PREC>;
     using Elem = typename TB::Elem;
     const int win = blockIdx.y, c = blockIdx.x, W = p.W;
@@ -297,6 +298,7 @@ __global__ void __launch_bounds__(OFF_THREADS) k_off_part(Params p, JoinScratch 
 // fixed order (lane by lane, then the lanes).
 __global__ void __launch_bounds__(256) k_off_fold(Params p, JoinScratch j, int nchunks)
 {
+    after_previous();
     const int win = blockIdx.x, W = p.W, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (!p.active[win]) return;
     const int ref = p.join_exclude == 0 ? 1 : 0;
@@ -328,6 +330,7 @@ __global__ void __launch_bounds__(256) k_off_fold(Params p, JoinScratch j, int n
 template <int PREC>
 __global__ void __launch_bounds__(256) k_merge(Params p, JoinScratch j)
 {
+    after_previous();
     using TB = tab::Tab<PREC>;
     using Elem = typename TB::Elem;
     extern __shared__ double s_off[];
@@ -382,6 +385,7 @@ __global__ void __launch_bounds__(256) k_merge(Params p, JoinScratch j)
 // (window, e).  (One thread each before: 514 -> 240 us at L = 32.)
 __global__ void __launch_bounds__(256) k_marg_piece(Params p, JoinScratch j)
 {
+    after_previous();
     const int idx = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (idx >= p.nwin * p.wE) return;
     const int win = idx / p.wE, el = idx % p.wE;
@@ -393,6 +397,7 @@ __global__ void __launch_bounds__(256) k_marg_piece(Params p, JoinScratch j)
 // chain is sequential; each matching point and slice rule is block-parallel).
 __global__ void __launch_bounds__(MATCH_THREADS) k_match_e(Params p, JoinScratch j)
 {
+    after_previous();
     const int b = blockIdx.x;
     if (b >= p.nM) return;
     const int nE = p.nE, t0 = threadIdx.x == 0;
@@ -482,6 +487,7 @@ constexpr int ROW_COLS = 8, ROW_ES = 32;
 
 __global__ void __launch_bounds__(ROW_COLS * ROW_ES) k_marg_row(Params p, JoinScratch j)
 {
+    after_previous();
     const int B = p.N + 1, b = blockIdx.y, cx = threadIdx.x % ROW_COLS, ex = threadIdx.x / ROW_COLS;
     const int m = (int)blockIdx.x * ROW_COLS + cx;
     __shared__ double s_part[ROW_ES][ROW_COLS];
@@ -522,6 +528,7 @@ __global__ void __launch_bounds__(ROW_COLS * ROW_ES) k_marg_row(Params p, JoinSc
 // chain, block-parallel matching point and slice rule).
 __global__ void __launch_bounds__(MATCH_THREADS) k_match_m(Params p, JoinScratch j)
 {
+    after_previous();
     const int nM = p.nM, nE = p.nE, B = p.N + 1, t0 = threadIdx.x == 0;
     __shared__ int s_first, s_last, s_bad;
     if (t0) {
@@ -574,6 +581,7 @@ constexpr int RED_BLOCKS = 512;     // red[]: 512 maxima (their order), then fro
 
 __global__ void __launch_bounds__(256) k_assemble(Params p, JoinScratch j)
 {
+    after_previous();
     const int B = p.N + 1;
     int mo = ORDER_NONE;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < (size_t)B * B; idx += (size_t)gridDim.x * blockDim.x) {
@@ -617,6 +625,7 @@ __device__ __forceinline__ int fold_max(const double *red, int n)
 
 __global__ void __launch_bounds__(256) k_red_sumexp(const double *v, size_t n, double *red, int nblk)
 {
+    after_previous();
     const int mo = fold_max(red, nblk);
     const double top = top_of(mo);
     double acc = 0.0;
@@ -639,6 +648,7 @@ __global__ void __launch_bounds__(256) k_red_sumexp(const double *v, size_t n, d
 
 __global__ void __launch_bounds__(256) k_normalise(double *v, size_t n, const double *red, int nblk, int N)
 {
+    after_previous();
     const double top = top_of(fold_max(red, nblk));
     double acc = 0.0;
     for (int k = threadIdx.x; k < nblk; k += 256) acc += red[RED_BLOCKS + k];
@@ -668,9 +678,9 @@ template <int PREC>
 void launch_merge(const Params &p, const JoinScratch &j, cudaStream_t s)
 {
     const int chunk = off_chunk(p), nchunks = (p.T + chunk - 1) / chunk;
-    k_off_part<PREC><<<dim3(nchunks, p.nwin), OFF_THREADS, 0, s>>>(p, j, chunk, nchunks);
-    if (nchunks > 1) k_off_fold<<<p.nwin, 256, 0, s>>>(p, j, nchunks);
-    k_merge<PREC><<<dim3((p.T + 511) / 512, p.nwin), 256, sizeof(double) * p.W, s>>>(p, j);
+    launch_next(k_off_part<PREC>, dim3(nchunks, p.nwin), dim3(OFF_THREADS), 0, s, p, j, chunk, nchunks);
+    if (nchunks > 1) launch_next(k_off_fold, dim3(p.nwin), dim3(256), 0, s, p, j, nchunks);
+    launch_next(k_merge<PREC>, dim3((p.T + 511) / 512, p.nwin), dim3(256), sizeof(double) * p.W, s, p, j);
 }
 
 }  // namespace
@@ -682,21 +692,22 @@ cudaError_t launch_join(const Params &p, const JoinScratch &j, cudaStream_t s)
     else if (p.precision == REWL_F32X2) launch_merge<REWL_F32X2>(p, j, s);
     else launch_merge<REWL_F32>(p, j, s);
     const int rows = p.nwin * p.wE, warps = row_warps(rows);
-    k_marg_piece<<<(rows + warps - 1) / warps, 32 * warps, 0, s>>>(p, j);
-    k_match_e<<<p.nM, MATCH_THREADS, 0, s>>>(p, j);
-    k_marg_row<<<dim3((B + ROW_COLS - 1) / ROW_COLS, p.nM), ROW_COLS * ROW_ES, 0, s>>>(p, j);
-    k_match_m<<<1, MATCH_THREADS, 0, s>>>(p, j);
+    launch_next(k_marg_piece, dim3((rows + warps - 1) / warps), dim3(32 * warps), 0, s, p, j);
+    launch_next(k_match_e, dim3(p.nM), dim3(MATCH_THREADS), 0, s, p, j);
+    launch_next(k_marg_row, dim3((B + ROW_COLS - 1) / ROW_COLS, p.nM), dim3(ROW_COLS * ROW_ES), 0, s, p, j);
+    launch_next(k_match_m, dim3(1), dim3(MATCH_THREADS), 0, s, p, j);
     const size_t nJ = (size_t)B * B;
     const int nblk = (int)std::min<size_t>(RED_BLOCKS, (nJ + 255) / 256);
-    k_assemble<<<nblk, 256, 0, s>>>(p, j);
-    k_red_sumexp<<<nblk, 256, 0, s>>>(j.J, nJ, j.red, nblk);
-    k_normalise<<<nblk, 256, 0, s>>>(j.J, nJ, j.red, nblk, p.N);
+    launch_next(k_assemble, dim3(nblk), dim3(256), 0, s, p, j);
+    launch_next(k_red_sumexp, dim3(nblk), dim3(256), 0, s, j.J, nJ, j.red, nblk);
+    launch_next(k_normalise, dim3(nblk), dim3(256), 0, s, j.J, nJ, j.red, nblk, p.N);
     return cudaGetLastError();
 }
 
 // Eq. 3 on the joined table: ln sum_m g(e, m), one warp per e.
 __global__ void __launch_bounds__(256) k_marg_out(Params p, JoinScratch j)
 {
+    after_previous();
     const int B = p.N + 1;
     const int e = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (e >= B) return;
@@ -707,7 +718,7 @@ __global__ void __launch_bounds__(256) k_marg_out(Params p, JoinScratch j)
 cudaError_t launch_marginal_e(const Params &p, const JoinScratch &j, cudaStream_t s)
 {
     const int rows = p.N + 1, warps = row_warps(rows);
-    k_marg_out<<<(rows + warps - 1) / warps, 32 * warps, 0, s>>>(p, j);
+    launch_next(k_marg_out, dim3((rows + warps - 1) / warps), dim3(32 * warps), 0, s, p, j);
     return cudaGetLastError();
 }
 
@@ -716,6 +727,7 @@ cudaError_t launch_marginal_e(const Params &p, const JoinScratch &j, cudaStream_
 // is missing (-inf) in any replicate is marked NaN in jk_ref.
 __global__ void k_jk_accum(Params p, JoinScratch j, const double *x, size_t n, int k, int32_t *fail)
 {
+    after_previous();
     if (blockIdx.x == 0 && threadIdx.x == 0 && p.st->join_error && *fail == 0) *fail = k << 8 | p.st->join_error;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const double v = x[i];
@@ -735,6 +747,7 @@ __global__ void k_jk_accum(Params p, JoinScratch j, const double *x, size_t n, i
 
 __global__ void k_jk_final(JoinScratch j, double *mean, double *err, size_t n, int W)
 {
+    after_previous();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const double r = j.jk_ref[i];
         if (isnan(r)) {
@@ -752,13 +765,13 @@ __global__ void k_jk_final(JoinScratch j, double *mean, double *err, size_t n, i
 cudaError_t launch_jk_accum(const Params &p, const JoinScratch &j, const double *x, size_t n, int k, int32_t *fail,
                             cudaStream_t s)
 {
-    k_jk_accum<<<256, 256, 0, s>>>(p, j, x, n, k, fail);
+    launch_next(k_jk_accum, dim3(256), dim3(256), 0, s, p, j, x, n, k, fail);
     return cudaGetLastError();
 }
 
 cudaError_t launch_jk_final(const JoinScratch &j, double *mean, double *err, size_t n, int W, cudaStream_t s)
 {
-    k_jk_final<<<256, 256, 0, s>>>(j, mean, err, n, W);
+    launch_next(k_jk_final, dim3(256), dim3(256), 0, s, j, mean, err, n, W);
     return cudaGetLastError();
 }
 

@@ -186,6 +186,7 @@ cudaError_t launch_drive(const Params &p, int32_t *d_fail, cudaStream_t s)
 template <int WPR, int PREC, bool REG>
 __global__ void __launch_bounds__(128) k_sweep_thread(Params p, unsigned long long ntrials)
 {
+    after_previous();
     using TB = Tab<PREC>;
     using Elem = typename TB::Elem;
     extern __shared__ uint32_t sm_all[];
@@ -399,6 +400,7 @@ cudaError_t launch_sweep_walker(const Params &p, int w, uint64_t ntrials, cudaSt
 // -> 14; L = 33, 5 walkers 25 -> 9.
 __global__ void __launch_bounds__(256) k_exchange(Params p)
 {
+    after_previous();
     extern __shared__ int perm[];              // W partners, then W draws / accepted flags
     int *const work = perm + p.W;
     __shared__ unsigned s_att, s_acc;
@@ -475,7 +477,7 @@ cudaError_t launch_exchange(const Params &p, int max_pairs, cudaStream_t s)
     if (max_pairs <= 0) return cudaSuccess;
     const long long tasks = (long long)p.W * p.nwords;
     const int threads = tasks <= 64 ? 64 : tasks <= 128 ? 128 : 256;
-    k_exchange<<<max_pairs, threads, 2 * (size_t)p.W * sizeof(int), s>>>(p);
+    launch_next(k_exchange, dim3(max_pairs), dim3(threads), 2 * (size_t)p.W * sizeof(int), s, p);
     return cudaGetLastError();
 }
 
@@ -498,6 +500,7 @@ struct FlatPart {
 template <bool SPLIT>
 __global__ void __launch_bounds__(256) k_flat(Params p)
 {
+    after_previous();
     if (p.st->done) return;
     namespace cg = cooperative_groups;
     const cg::cluster_group cl = cg::this_cluster();
@@ -548,7 +551,7 @@ cudaError_t launch_flat(const Params &p, cudaStream_t s)
     int parts = 1;
     while (parts < 8 && (long long)p.nwalk * parts < 152 * 4 && p.T / (2 * parts) >= 8192) parts *= 2;
     if (parts == 1) {
-        k_flat<false><<<p.nwalk, 256, 0, s>>>(p);
+        launch_next(k_flat<false>, dim3(p.nwalk), dim3(256), 0, s, p);
         return cudaGetLastError();
     }
     cudaLaunchConfig_t lc = {};
@@ -573,6 +576,7 @@ cudaError_t launch_flat(const Params &p, cudaStream_t s)
 // ln f <= lnf_final (Sec. 2: all walkers move on together; stop at f_final).
 __global__ void k_decide(Params p, int flags)
 {
+    after_previous();
     DevState *st = p.st;
     if (st->done) { st->advanced = 0; return; }
     if (flags & DECIDE_XSTEP) st->xstep += 1ull;
@@ -594,7 +598,7 @@ __global__ void k_decide(Params p, int flags)
 
 cudaError_t launch_decide(const Params &p, int flags, cudaStream_t s)
 {
-    k_decide<<<1, 1, 0, s>>>(p, flags);
+    launch_next(k_decide, dim3(1), dim3(1), 0, s, p, flags);
     return cudaGetLastError();
 }
 
@@ -609,6 +613,7 @@ cudaError_t launch_decide(const Params &p, int flags, cudaStream_t s)
 template <int PREC>
 __global__ void __launch_bounds__(256) k_fold(Params p, int fold)
 {
+    after_previous();
     using TB = Tab<PREC>;
     using Elem = typename TB::Elem;
     if (fold && !p.st->advanced) return;
@@ -653,9 +658,9 @@ __global__ void __launch_bounds__(256) k_fold(Params p, int fold)
 cudaError_t launch_fold(const Params &p, int fold, cudaStream_t s)
 {
     if (p.nwalk <= 0) return cudaSuccess;
-    if (p.precision == REWL_FP64) k_fold<REWL_FP64><<<p.nwalk, 256, 0, s>>>(p, fold);
-    else if (p.precision == REWL_F32X2) k_fold<REWL_F32X2><<<p.nwalk, 256, 0, s>>>(p, fold);
-    else k_fold<REWL_F32><<<p.nwalk, 256, 0, s>>>(p, fold);
+    if (p.precision == REWL_FP64) launch_next(k_fold<REWL_FP64>, dim3(p.nwalk), dim3(256), 0, s, p, fold);
+    else if (p.precision == REWL_F32X2) launch_next(k_fold<REWL_F32X2>, dim3(p.nwalk), dim3(256), 0, s, p, fold);
+    else launch_next(k_fold<REWL_F32>, dim3(p.nwalk), dim3(256), 0, s, p, fold);
     return cudaGetLastError();
 }
 

@@ -172,6 +172,7 @@ struct TreeShape {
 template <bool SMT, int G, int PREC, bool REG, bool WIDE>
 __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, int smem_per_walker)
 {
+    after_previous();
     using TB = Tab<PREC>;
     using Elem = typename TB::Elem;
     constexpr int DEPTH = TreeShape<G>::DEPTH;
@@ -676,8 +677,7 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kern<<<blocks, threads, smem, s>>>(p, (unsigned)ntrials, (int)per);
-        return cudaGetLastError();
+        return launch_next(kern, dim3(blocks), dim3(threads), smem, s, p, (unsigned)ntrials, (int)per);
     };
     const bool wide = blocks_of(p.L).n > 1;
 #define REWL_TREE_G(S_, P_, R_, W_)                                   \
