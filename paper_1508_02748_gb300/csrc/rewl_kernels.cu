@@ -676,6 +676,14 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z)
     return z ^ (z >> 31);
 }
 
+// of a 32-bit number
+__device__ __forceinline__ unsigned long long mix32(uint32_t i)
+{
+    unsigned long long z = (unsigned long long)(i ^ (i >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+
 // The bits of an entry's ln g.  The FP64 pipe is the scarce unit here (two
 // lanes an SM and cycle), and a bin without a visit in this iteration holds
 // its base, most of them 0, whose bits need none of it; the others are formed
@@ -710,7 +718,7 @@ __device__ __forceinline__ unsigned long long lng_bits(typename Tab<PREC>::Elem 
 // 64-bit division per entry before, every value formed in FP64).
 constexpr int DIGEST_CHUNK = 8192;
 
-template <int PREC>
+template <int PREC, bool SMALL>     // SMALL: fewer than 2^32 entries
 __global__ void __launch_bounds__(256) k_digest(Params p, int chunks, unsigned long long *out)
 {
     using Elem = typename Tab<PREC>::Elem;
@@ -724,7 +732,9 @@ __global__ void __launch_bounds__(256) k_digest(Params p, int chunks, unsigned l
     unsigned long long acc = 0;
     auto add = [&](int b, Elem v, int hv) {
         const unsigned long long i = w * p.T + (size_t)b, h = (unsigned long long)(uint32_t)hv;
-        acc += mix64(lng_bits<PREC>(v, hv, lnf) ^ mix64(i)) + mix64(h + 0x9E3779B97F4A7C15ull * i);
+        const unsigned long long mi = SMALL ? mix32((uint32_t)i) : mix64(i);
+        const unsigned long long gi = SMALL ? 0x9E3779B97F4A7C15ull * (uint32_t)i : 0x9E3779B97F4A7C15ull * i;
+        acc += mix64(lng_bits<PREC>(v, hv, lnf) ^ mi) + mix64(h + gi);
     };
     struct __align__(16) Four { Elem v[4]; };
     for (int b = b0 + 4 * (int)threadIdx.x; b < b1; b += 4 * 256) {
@@ -753,9 +763,11 @@ cudaError_t launch_digest(const Params &p, unsigned long long *d_out, cudaStream
 {
     const int chunks = (p.T + DIGEST_CHUNK - 1) / DIGEST_CHUNK;
     const unsigned blocks = (unsigned)p.nwalk * (unsigned)chunks;
-    if (p.precision == REWL_FP64) k_digest<REWL_FP64><<<blocks, 256, 0, s>>>(p, chunks, d_out);
-    else if (p.precision == REWL_F32X2) k_digest<REWL_F32X2><<<blocks, 256, 0, s>>>(p, chunks, d_out);
-    else k_digest<REWL_F32><<<blocks, 256, 0, s>>>(p, chunks, d_out);
+    auto go = [&](auto kern) { kern<<<blocks, 256, 0, s>>>(p, chunks, d_out); };
+    const bool small = (unsigned long long)p.nwalk * (unsigned long long)p.T < 1ull << 32;
+    if (p.precision == REWL_FP64) small ? go(k_digest<REWL_FP64, true>) : go(k_digest<REWL_FP64, false>);
+    else if (p.precision == REWL_F32X2) small ? go(k_digest<REWL_F32X2, true>) : go(k_digest<REWL_F32X2, false>);
+    else small ? go(k_digest<REWL_F32, true>) : go(k_digest<REWL_F32, false>);
     return cudaGetLastError();
 }
 
