@@ -47,9 +47,8 @@
 //
 // The outcome is the sequential chain itself, trial for trial:
 //   - random numbers are drawn per trial index from the TRIAL stream of
-//     Philox4x32-10, independent of the state (a ring of 128 trials per
-//     walker, refilled 64 at a time from the even trial at or below the
-//     launch's first trial);
+//     Philox4x32-10, independent of the state (a ring per walker,
+//     refilled from the even trial at or below the launch's first trial);
 //   - base(b) + n ln f is evaluated exactly in double (fma; the compensated
 //     pair converts exactly) and equals the sequential additions whenever
 //     ln f = 2^-k and the values stay within 53 (pair: 48) bits;
@@ -76,13 +75,15 @@
 // comparisons, the leaf by shuffle instead of a mailbox, the trial read a step
 // ahead and near-ties looked at on the path alone took 266-302 instructions a
 // step to 150.  Sampling launches of 10^4 trials per walker, GB300, 2070 MHz,
-// before -> after: L = 8 (36 walkers, 32 lanes, staged) 0.72 -> 0.37 ms; L = 16
+// before -> after: L = 8 (36 walkers, 32 lanes, staged) 0.72 -> 0.36 ms; L = 16
 // (256 walkers, 32 lanes) 0.95 -> 0.64 ms; L = 32 (2048 walkers, 32 lanes) 1.64
 // -> 1.05 ms; L = 64 (3904 walkers, 16 lanes) 2.71 -> 1.60 ms.
 // Tried and slower: the visits of recent bins in a shared-memory cache (L1
 // loses the space), prefetching the neighbourhood's lines (its instructions
 // cost what it saves), the path's end by a warp reduction, flips or stores
 // under a branch.
+#include <type_traits>
+
 #include "rewl_tab.cuh"
 
 namespace rewl {
@@ -91,7 +92,11 @@ using namespace tab;
 
 namespace {
 
-constexpr int RING = 128;   // trials buffered per walker
+// Trials drawn per refill of a walker's ring, which holds two refills.  With a
+// whole warp for a walker whose tables are staged (few walkers) a refill's
+// latency counts, and two Philox calls a lane at once take hardly longer than
+// one (L = 8, 36 walkers: 0.370 -> 0.357 ms); else its shared memory does.
+__host__ __device__ constexpr int chunk_of(bool staged, int G) { return staged && G == 32 ? 128 : 64; }
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
 // The lattice in shared memory: each row is cut into nblk blocks of at most
@@ -134,9 +139,14 @@ struct RingEntry {
     float lnu;     // ln u in float
 };
 static_assert(sizeof(RingEntry) == 16, "one vector load per trial");
-constexpr size_t RING_BYTES = (RING + RING_TAIL) * sizeof(RingEntry);
+__host__ __device__ constexpr size_t ring_bytes(bool staged, int G)
+{
+    return (2 * chunk_of(staged, G) + RING_TAIL) * sizeof(RingEntry);
+}
+
 // Register lattice: each trial's site as a 64-bit mask, beside the ring.
-constexpr size_t BITS_BYTES = (RING + RING_TAIL) * sizeof(uint2);
+__host__ __device__ constexpr size_t bits_bytes(bool staged, int G) { return ring_bytes(staged, G) / 2; }
+static_assert(2 * sizeof(uint2) == sizeof(RingEntry), "half a ring entry");
 
 // Eq. 1 decided from the exact values (near-ties of the float screen on the
 // true path only).
@@ -165,11 +175,11 @@ struct TreeShape {
 
 }  // namespace
 
-// REG: the lattice (N <= 64 sites, bit i*L + j) is held in a 64-bit register
-// by every lane; otherwise it lives in shared memory (Blocks).  SMT: S and H
-// staged in shared memory for the launch.
-// WIDE: rows of several blocks.
-template <bool SMT, int G, int PREC, bool REG, bool WIDE>
+// LAT: the lattice (N <= 32 or N <= 64 sites, bit i*L + j) is held in one or two
+// registers by every lane (LAT = 1, 2); otherwise it lives in shared memory
+// (Blocks), its rows one block each (0) or several (3).  SMT: S and H staged in
+// shared memory for the launch.
+template <bool SMT, int G, int PREC, int LAT>
 __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, int smem_per_walker)
 {
     after_previous();
@@ -178,6 +188,9 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
     constexpr int DEPTH = TreeShape<G>::DEPTH;
     constexpr int GPW = 32 / G;   // walkers per warp
     constexpr unsigned GBITS = G == 32 ? 0xFFFFFFFFu : ((1u << G) - 1u);
+    constexpr bool REG = LAT == 1 || LAT == 2, HI = LAT == 2, WIDE = LAT == 3;
+    constexpr int CHUNK = chunk_of(SMT, G), RING = 2 * CHUNK;
+    constexpr size_t RING_BYTES = ring_bytes(SMT, G), BITS_BYTES = bits_bytes(SMT, G);
     constexpr unsigned RMASK = RING - 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -337,11 +350,11 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
     int err = 0;                    // sign: a count passed INT_MAX
 
     while (u < ntrials) {
-        // ---- refill the ring: 32 Philox calls = 64 trials (the test leaves
-        // the parity of t0 out, so the warp's groups refill together)
-        if (2 * cfill < u + 33) {
-            #pragma unroll 1
-            for (int r = 0; r < 32 / G; ++r) {
+        // ---- refill the ring (the test leaves the parity of t0 out, so the
+        // warp's groups refill together)
+        if (2 * cfill < u + CHUNK / 2 + 1) {
+            #pragma unroll (CHUNK == 128 ? 2 : 1)
+            for (int r = 0; r < CHUNK / 2 / G; ++r) {
                 const unsigned long long c = c0 + cfill + (unsigned)(gl + r * G);
                 const u32x4 x = philox10((uint32_t)c, (uint32_t)(c >> 32), (uint32_t)w, TAG_TRIAL, p.key0, p.key1);
                 #pragma unroll
@@ -393,9 +406,9 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
             }
             __syncwarp();
             if (!REG) {
-                // relation codes of the 64 new trials to the DEPTH trials before each
+                // relation codes of the new trials to the DEPTH trials before each
                 #pragma unroll 1
-                for (int r = 0; r < 64 / G; ++r) {
+                for (int r = 0; r < CHUNK / G; ++r) {
                     const unsigned q = (unsigned)(2 * (c0 + cfill)) + (unsigned)(gl + r * G);
                     const unsigned at = q & RMASK;
                     const uint32_t b = ring[at].b, site = b >> 20;
@@ -416,7 +429,7 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
                     if (at < RING_TAIL) ring[at + RING].b = rel;
                 }
             }
-            cfill += 32;
+            cfill += CHUNK / 2;
             __syncwarp();
         }
         // steps until the ring runs low or the launch ends; its last step may
@@ -443,7 +456,7 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
                 for (int k = 0; k < DEPTH; ++k) {
                     const uint2 b = bits[now + k];
                     nlo ^= b.x & flip[k];
-                    nhi ^= b.y & flip[k];
+                    if (HI) nhi ^= b.y & flip[k];
                 }
                 nbit = bits[now + dl];
             }
@@ -457,11 +470,16 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
         int pk;
         if (REG) {
             hlo = lo ^ nlo;
-            hhi = hi ^ nhi;
             olo = nbit.x;
-            ohi = nbit.y;
-            const bool sup = ((hlo & olo) | (hhi & ohi)) != 0u;
-            pk = (__popc(hlo & me.a) + __popc(hhi & me.b)) * (sup ? mvA : -mvA) + (sup ? -mvB : mvB);
+            bool sup = (hlo & olo) != 0u;
+            int nup = __popc(hlo & me.a);
+            if (HI) {
+                hhi = hi ^ nhi;
+                ohi = nbit.y;
+                sup = ((hlo & olo) | (hhi & ohi)) != 0u;
+                nup += __popc(hhi & me.b);
+            }
+            pk = nup * (sup ? mvA : -mvA) + (sup ? -mvB : mvB);
         } else {
             const uint32_t wc = lat[(me.a >> 8) & 0xFFu], wu = lat[(me.a >> 16) & 0xFFu], wd = lat[me.a >> 24];
             uint32_t v5 = (__funnelshift_r(wc, wc, me.a) & 7u) | (__funnelshift_r(wu, wu, me.a - 2u) & 8u)
@@ -538,7 +556,7 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
             Pa = __shfl_sync(FULL, acc ? Pn : Pc, leaf);
             if (REG) {
                 lo2 = __shfl_sync(FULL, acc ? hlo ^ olo : hlo, leaf);
-                hi2 = __shfl_sync(FULL, acc ? hhi ^ ohi : hhi, leaf);
+                if (HI) hi2 = __shfl_sync(FULL, acc ? hhi ^ ohi : hhi, leaf);
             }
             path = __shfl_sync(FULL, acc ? hacc : hist, leaf);   // bit k: trial k accepted
         };
@@ -640,7 +658,7 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
 size_t tree_smem_per_warp(const Params &p, bool smt, int group)
 {
     const size_t nlat = (size_t)p.L * blocks_of(p.L).n + group;
-    size_t b = RING_BYTES + (p.lattice_reg ? BITS_BYTES : (nlat * 4 + 15) & ~(size_t)15);
+    size_t b = ring_bytes(smt, group) + (p.lattice_reg ? bits_bytes(smt, group) : (nlat * 4 + 15) & ~(size_t)15);
     if (smt) b += (size_t)(p.wE + 4) * staged_ld(p.wM) * 8;
     return (b + 15) & ~(size_t)15;
 }
@@ -657,7 +675,7 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
     // a window whose bins fit in a block's shared memory, but not with the
     // entries around them, is sampled from global memory
     if (smt && tree_smem_per_warp(p, true, group) * gpw > max_smem
-        && (RING * sizeof(RingEntry) + 48 + (((size_t)p.nwords * 4 + 15) & ~(size_t)15) + 8 * (size_t)p.T) * gpw <= max_smem)
+        && (128 * sizeof(RingEntry) + 48 + (((size_t)p.nwords * 4 + 15) & ~(size_t)15) + 8 * (size_t)p.T) * gpw <= max_smem)
         smt = false;
     const size_t per = tree_smem_per_warp(p, smt, group);
     // one warp a block: blocks of several warps leave when their last walker
@@ -679,23 +697,25 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
         }
         return launch_next(kern, dim3(blocks), dim3(threads), smem, s, p, (unsigned)ntrials, (int)per);
     };
-    const bool wide = blocks_of(p.L).n > 1;
-#define REWL_TREE_G(S_, P_, R_, W_)                                   \
-    if (group == 32) return go(k_sweep_tree<S_, 32, P_, R_, W_>);     \
-    if (group == 16) return go(k_sweep_tree<S_, 16, P_, R_, W_>);     \
-    return go(k_sweep_tree<S_, 8, P_, R_, W_>);
-#define REWL_TREE_R(S_, P_)                                           \
-    if (p.lattice_reg) { REWL_TREE_G(S_, P_, true, false) }           \
-    if (wide) { REWL_TREE_G(S_, P_, false, true) }                    \
-    REWL_TREE_G(S_, P_, false, false)
-    if (p.precision == REWL_FP64) {
-        if (smt) { REWL_TREE_R(true, REWL_FP64) }
-        REWL_TREE_R(false, REWL_FP64)
-    }
-    if (smt) { REWL_TREE_R(true, REWL_F32X2) }
-    REWL_TREE_R(false, REWL_F32X2)
-#undef REWL_TREE_R
-#undef REWL_TREE_G
+    const int lat = p.lattice_reg ? (p.N <= 32 ? 1 : 2) : blocks_of(p.L).n > 1 ? 3 : 0;
+    auto with = [&](auto staged, auto g, auto prec) -> cudaError_t {
+        constexpr bool S = decltype(staged)::value;
+        constexpr int G = decltype(g)::value, P = decltype(prec)::value;
+        if (lat == 1) return go(k_sweep_tree<S, G, P, 1>);
+        if (lat == 2) return go(k_sweep_tree<S, G, P, 2>);
+        if (lat == 3) return go(k_sweep_tree<S, G, P, 3>);
+        return go(k_sweep_tree<S, G, P, 0>);
+    };
+    auto lanes = [&](auto staged, auto prec) -> cudaError_t {
+        if (group == 32) return with(staged, std::integral_constant<int, 32>(), prec);
+        if (group == 16) return with(staged, std::integral_constant<int, 16>(), prec);
+        return with(staged, std::integral_constant<int, 8>(), prec);
+    };
+    auto tables = [&](auto prec) -> cudaError_t {
+        return smt ? lanes(std::true_type(), prec) : lanes(std::false_type(), prec);
+    };
+    return p.precision == REWL_FP64 ? tables(std::integral_constant<int, REWL_FP64>())
+                                    : tables(std::integral_constant<int, REWL_F32X2>());
 }
 
 }  // namespace rewl
