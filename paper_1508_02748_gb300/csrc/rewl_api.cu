@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -37,9 +38,47 @@ struct rewl_s {
     cudaStream_t plain_s[REWL_PLAIN_STREAMS];
     cudaEvent_t plain_ev[REWL_PLAIN_STREAMS + 1];
     bool plain_ok;
+    unsigned char *pin;              // kPinBytes of pinned host memory for small results, null if none was to be had
 };
 
 namespace {
+
+// Pinned host memory for the small results of a call (state, matching points):
+// copies into it are queued behind the work and share one wait, where a copy
+// into pageable memory waits by itself.  A handle holds one block from creation
+// to destruction; up to kPinKept returned blocks are kept for the next handles.
+constexpr size_t kPinBytes = 16 * 1024;
+constexpr int kPinKept = 32;
+std::mutex g_pin_mu;
+unsigned char *g_pin_free[kPinKept];
+int g_pin_n = 0;
+
+unsigned char *pin_take()
+{
+    {
+        std::lock_guard<std::mutex> lk(g_pin_mu);
+        if (g_pin_n > 0) return g_pin_free[--g_pin_n];
+    }
+    void *b = nullptr;
+    if (cudaHostAlloc(&b, kPinBytes, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();          // (then results are copied one by one)
+        return nullptr;
+    }
+    return (unsigned char *)b;
+}
+
+void pin_give(unsigned char *b)
+{
+    if (!b) return;
+    {
+        std::lock_guard<std::mutex> lk(g_pin_mu);
+        if (g_pin_n < kPinKept) {
+            g_pin_free[g_pin_n++] = b;
+            return;
+        }
+    }
+    cudaFreeHost(b);
+}
 
 const char *g_noerr = "";
 char g_create_err[512];
@@ -281,23 +320,67 @@ int sync(rewl_t *h)
     return REWL_OK;
 }
 
+// Small results fetched together: add() queues a copy behind the work on the
+// run's stream, wait() waits once, give() hands the bytes out.  add() is false
+// where there is no room in pinned memory: such a result is copied by itself.
+struct Fetch {
+    rewl_t *h;
+    size_t used = 0;
+    int n = 0;
+    struct { void *to; size_t at, bytes; } part[4];
+    cudaError_t err = cudaSuccess;
+
+    explicit Fetch(rewl_t *handle) : h(handle) {}
+    bool add(void *to, const void *dev, size_t bytes)
+    {
+        const size_t at = (used + 15) & ~(size_t)15;
+        if (!h->pin || n == 4 || at + bytes > kPinBytes || at + bytes < bytes) return false;
+        if (err == cudaSuccess) err = cudaMemcpyAsync(h->pin + at, dev, bytes, cudaMemcpyDeviceToHost, h->stream);
+        part[n++] = {to, at, bytes};
+        used = at + bytes;
+        return true;
+    }
+    // one of the few words every call needs
+    void need(void *to, const void *dev, size_t bytes)
+    {
+        if (!add(to, dev, bytes) && err == cudaSuccess)
+            err = cudaMemcpyAsync(to, dev, bytes, cudaMemcpyDeviceToHost, h->stream);
+    }
+    cudaError_t wait()
+    {
+        if (err == cudaSuccess) err = cudaStreamSynchronize(h->stream);
+        return err;
+    }
+    void give(int from = 0)
+    {
+        for (int i = from; i < n; ++i) std::memcpy(part[i].to, h->pin + part[i].at, part[i].bytes);
+    }
+};
+
 int read_state(rewl_t *h, DevState *ds)
 {
-    CK(h, cudaMemcpyAsync(ds, h->p.st, sizeof(DevState), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
+    Fetch f(h);
+    f.need(ds, h->p.st, sizeof(DevState));
+    CK(h, f.wait());
+    f.give();
     if (ds->error & ERR_OVERFLOW) return fail(h, REWL_E_OVERFLOW, "histogram entry above INT32_MAX");
     return REWL_OK;
 }
 
-unsigned long long trials_of(rewl_t *h)
+// The state and, for a status, the trials of the first walker that samples.
+int read_status(rewl_t *h, DevState *ds, unsigned long long *trials)
 {
-    unsigned long long t = 0;
-    if (h->first_active < 0) return 0;
-    if (cudaMemcpy(&t, h->p.wt + h->first_active, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return 0;
-    return t;
+    *trials = 0;
+    Fetch f(h);
+    f.need(ds, h->p.st, sizeof(DevState));
+    if (h->first_active >= 0) f.need(trials, h->p.wt + h->first_active, 8);
+    CK(h, f.wait());
+    f.give();
+    if (ds->error & ERR_OVERFLOW) return fail(h, REWL_E_OVERFLOW, "histogram entry above INT32_MAX");
+    return REWL_OK;
 }
 
-void fill_status(rewl_t *h, const DevState &ds, rewl_status *s)
+void fill_status(rewl_t *h, const DevState &ds, unsigned long long trials, rewl_status *s)
 {
     if (!s) return;
     std::memset(s, 0, sizeof(*s));
@@ -305,7 +388,7 @@ void fill_status(rewl_t *h, const DevState &ds, rewl_status *s)
     s->done = ds.done;
     s->lnf = ds.lnf;
     s->cycles = ds.cycle;
-    s->trials = trials_of(h);
+    s->trials = trials;
     s->exch_attempts = ds.exch_attempts;
     s->exch_accepts = ds.exch_accepts;
     s->n_flat = ds.nflat_last;
@@ -403,6 +486,7 @@ int create_impl(const rewl_config *cfg, const uint8_t *host_init_spins, void *d_
     h->host_cycle = 0;
     h->wpb = cfg->walkers_per_block;
     h->graph_ok = false;
+    h->pin = pin_take();
     h->max_pairs = max_pairs_of(d);
 
     char *base = (char *)d_workspace;
@@ -668,9 +752,10 @@ extern "C" int rewl_run_cycles(rewl_t *h, uint64_t n_cycles, rewl_status *status
     int rc = queue_cycles(h, n_cycles);
     if (rc) return rc;
     DevState ds;
-    rc = read_state(h, &ds);
+    unsigned long long trials;
+    rc = read_status(h, &ds, &trials);
     if (rc) return rc;
-    fill_status(h, ds, status);
+    fill_status(h, ds, trials, status);
     return REWL_OK;
 }
 
@@ -729,9 +814,10 @@ extern "C" int rewl_run_cycles_plain(rewl_t *h, uint64_t n_cycles, rewl_status *
         if (rc) return rc;
     }
     DevState ds;
-    int rc = read_state(h, &ds);
+    unsigned long long trials;
+    const int rc = read_status(h, &ds, &trials);
     if (rc) return rc;
-    fill_status(h, ds, status);
+    fill_status(h, ds, trials, status);
     return REWL_OK;
 }
 
@@ -739,10 +825,11 @@ extern "C" int rewl_run_iteration(rewl_t *h, uint64_t max_cycles, rewl_status *s
 {
     if (!h) return REWL_E_INVALID;
     DevState ds;
-    int rc = read_state(h, &ds);
+    unsigned long long trials;
+    int rc = read_status(h, &ds, &trials);
     if (rc) return rc;
     const int it0 = ds.iter;
-    if (ds.done) { fill_status(h, ds, status); return REWL_OK; }
+    if (ds.done) { fill_status(h, ds, trials, status); return REWL_OK; }
     uint64_t ran = 0;
     const uint64_t ce = (uint64_t)h->cfg.check_every;
     while (ran < max_cycles) {
@@ -752,11 +839,11 @@ extern "C" int rewl_run_iteration(rewl_t *h, uint64_t max_cycles, rewl_status *s
         rc = queue_cycles(h, n);
         if (rc) return rc;
         ran += n;
-        rc = read_state(h, &ds);
+        rc = read_status(h, &ds, &trials);
         if (rc) return rc;
-        if (ds.done || ds.iter != it0) { fill_status(h, ds, status); return REWL_OK; }
+        if (ds.done || ds.iter != it0) { fill_status(h, ds, trials, status); return REWL_OK; }
     }
-    fill_status(h, ds, status);
+    fill_status(h, ds, trials, status);
     return fail(h, REWL_E_BUDGET, "no iteration ended within %llu cycles", (unsigned long long)max_cycles);
 }
 
@@ -793,9 +880,10 @@ extern "C" int rewl_get_status(rewl_t *h, rewl_status *status)
 {
     if (!h || !status) return REWL_E_INVALID;
     DevState ds;
-    int rc = read_state(h, &ds);
+    unsigned long long trials;
+    const int rc = read_status(h, &ds, &trials);
     if (rc) return rc;
-    fill_status(h, ds, status);
+    fill_status(h, ds, trials, status);
     return REWL_OK;
 }
 
@@ -971,17 +1059,23 @@ extern "C" int rewl_get_lng(rewl_t *h, int what, double *host_out, size_t capaci
     CK(h, cudaMemsetAsync(&p.st->join_error, 0, sizeof(int32_t), h->stream));
     CK(h, launch_join(p, h->j, h->stream));
     if (what == REWL_LNG_MARGINAL_E) CK(h, launch_marginal_e(p, h->j, h->stream));
+    const size_t em_bytes = 4 * (size_t)p.nM * (p.nE > 1 ? p.nE - 1 : 1), mm_bytes = 4 * (size_t)(p.nM > 1 ? p.nM - 1 : 1);
     DevState ds;
-    int rc = read_state(h, &ds);
-    if (rc) return rc;
+    Fetch f(h);
+    f.need(&ds, p.st, sizeof(DevState));
+    const int states = f.n;
+    const bool em = host_ematch && f.add(host_ematch, h->j.ematch, em_bytes);
+    const bool mm = host_mmatch && f.add(host_mmatch, h->j.mmatch, mm_bytes);
+    CK(h, f.wait());
+    if (states) std::memcpy(&ds, h->pin, sizeof(DevState));
+    if (ds.error & ERR_OVERFLOW) return fail(h, REWL_E_OVERFLOW, "histogram entry above INT32_MAX");
     if (ds.join_error) return fail(h, REWL_E_JOIN, "join failed (code %d): adjacent pieces share no visited bins", ds.join_error);
+    f.give(states);
     CK(h, cudaMemcpyAsync(host_out, what == REWL_LNG_JOINED ? h->j.J : h->j.marg, 8 * n, cudaMemcpyDeviceToHost, h->stream));
-    if (host_ematch)
-        CK(h, cudaMemcpyAsync(host_ematch, h->j.ematch, 4 * (size_t)p.nM * (p.nE > 1 ? p.nE - 1 : 1),
-                              cudaMemcpyDeviceToHost, h->stream));
-    if (host_mmatch)
-        CK(h, cudaMemcpyAsync(host_mmatch, h->j.mmatch, 4 * (size_t)(p.nM > 1 ? p.nM - 1 : 1),
-                              cudaMemcpyDeviceToHost, h->stream));
+    if (host_ematch && !em)
+        CK(h, cudaMemcpyAsync(host_ematch, h->j.ematch, em_bytes, cudaMemcpyDeviceToHost, h->stream));
+    if (host_mmatch && !mm)
+        CK(h, cudaMemcpyAsync(host_mmatch, h->j.mmatch, mm_bytes, cudaMemcpyDeviceToHost, h->stream));
     return sync(h);
 }
 
@@ -1013,10 +1107,13 @@ extern "C" int rewl_get_lng_jackknife(rewl_t *h, int what, double *host_mean, do
     }
     CK(h, launch_jk_final(h->j, h->jk_mean, h->jk_err, n, p.W, h->stream));
     int32_t failed = 0;
-    CK(h, cudaMemcpyAsync(&failed, h->d_fail, sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
     DevState ds;
-    const int rc = read_state(h, &ds);
-    if (rc) return rc;
+    Fetch f(h);
+    f.need(&failed, h->d_fail, sizeof(int32_t));
+    f.need(&ds, h->p.st, sizeof(DevState));
+    CK(h, f.wait());
+    f.give();
+    if (ds.error & ERR_OVERFLOW) return fail(h, REWL_E_OVERFLOW, "histogram entry above INT32_MAX");
     if (failed)
         return fail(h, REWL_E_JOIN, "jackknife replicate %d: join failed (code %d)", failed >> 8, failed & 0xFF);
     CK(h, cudaMemcpyAsync(host_mean, h->jk_mean, 8 * n, cudaMemcpyDeviceToHost, h->stream));
@@ -1038,6 +1135,7 @@ extern "C" int rewl_destroy(rewl_t *h)
         for (int i = 0; i < REWL_PLAIN_STREAMS; ++i) cudaStreamDestroy(h->plain_s[i]);
         for (int i = 0; i <= REWL_PLAIN_STREAMS; ++i) cudaEventDestroy(h->plain_ev[i]);
     }
+    pin_give(h->pin);
     delete h;
     return REWL_OK;
 }

@@ -108,6 +108,8 @@ _lock = threading.Lock()
 def load_library(path: str | None = None):
     """Loads librewl.so (built by ``paper_1508_02748_gb300.build``); raises if absent."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             p = path or LIB_PATH
@@ -380,9 +382,9 @@ def relative_difference(lng_a, lng_b) -> "object":
         raise ValueError("two float64 CUDA tensors of one shape on one device expected")
     out = torch.empty_like(a)
     s = torch.cuda.current_stream(a.device)
-    _check(load_library().rewl_relative_difference(ctypes.c_void_p(a.data_ptr()), ctypes.c_void_p(b.data_ptr()),
-                                                   ctypes.c_void_p(out.data_ptr()), a.numel(),
-                                                   ctypes.c_void_p(s.cuda_stream)))
+    rc = load_library().rewl_relative_difference(a.data_ptr(), b.data_ptr(), out.data_ptr(), a.numel(), s.cuda_stream)
+    if rc:
+        _check(rc)
     return out
 
 
