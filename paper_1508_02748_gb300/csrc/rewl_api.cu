@@ -311,6 +311,7 @@ void choose_tiling(rewl_t *h, long long walkers)
     else if (c.table_mode != REWL_TABLES_AUTO) p.smt = c.table_mode == REWL_TABLES_STAGED;
     else p.smt = block * (blocks ? blocks : 1) <= kSmem + kPerBlock;
     p.group = p.smt ? staged_lanes : global_lanes;
+    p.sharing = walkers;
     if (c.lattice_mode == REWL_LATTICE_AUTO && !p.smt && p.group != 8) p.lattice_reg = 0;
 }
 

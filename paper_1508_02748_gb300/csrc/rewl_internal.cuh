@@ -73,6 +73,7 @@ struct Params {
     int sampler;      // REWL_SAMPLER_WARP or REWL_SAMPLER_THREAD
     int smt;          // warp sampler: tables staged in shared memory
     int group;        // warp sampler: lanes per walker
+    long long sharing;// warp sampler: walkers that share the GPU with this run's, its own among them
     int lattice_reg;  // warp sampler: the lattice in a 64-bit register (N <= 64)
     uint32_t key0, key1;
     uint32_t divL;    // ceil(2^32 / L): site / L = umulhi(site, divL) for site < N
@@ -137,20 +138,34 @@ struct JoinScratch {
 // ten short kernels: L = 8 137 -> 116 us, L = 16's jackknife 5.8 -> 5.15 ms.
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// carveout: percent of an SM's memory that shared memory is to have, -1 for the
+// driver's choice.
 template <class... P, class... A>
-inline cudaError_t launch_next(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+inline cudaError_t launch_next_with(int carveout, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                    A... args)
 {
     cudaLaunchConfig_t lc = {};
     lc.gridDim = grid;
     lc.blockDim = block;
     lc.dynamicSmemBytes = smem;
     lc.stream = s;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = &at;
-    lc.numAttrs = s != nullptr ? 1 : 0;
+    cudaLaunchAttribute at[2];
+    lc.attrs = at;
+    if (s != nullptr) {
+        at[lc.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[lc.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (carveout >= 0) {
+        at[lc.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        at[lc.numAttrs++].val.sharedMemCarveout = (unsigned)carveout;
+    }
     return cudaLaunchKernelEx(&lc, kernel, P(args)...);
+}
+
+template <class... P, class... A>
+inline cudaError_t launch_next(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    return launch_next_with(-1, kernel, grid, block, smem, s, args...);
 }
 
 // Kernel launchers (rewl_kernels.cu, rewl_join.cu); all return cudaError_t of the launch.

@@ -82,6 +82,7 @@
 // loses the space), prefetching the neighbourhood's lines (its instructions
 // cost what it saves), the path's end by a warp reduction, flips or stores
 // under a branch.
+#include <algorithm>
 #include <type_traits>
 
 #include "rewl_tab.cuh"
@@ -357,12 +358,15 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
             for (int r = 0; r < CHUNK / 2 / G; ++r) {
                 const unsigned long long c = c0 + cfill + (unsigned)(gl + r * G);
                 const u32x4 x = philox10((uint32_t)c, (uint32_t)(c >> 32), (uint32_t)w, TAG_TRIAL, p.key0, p.key1);
+                uint32_t si[2], sj[2];
                 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
                     const uint32_t xs = hh ? x.z : x.x, xu = hh ? x.w : x.y;
                     const uint32_t site = __umulhi(xs, N);
                     const uint32_t i = __umulhi(site, divL);
                     const uint32_t j = site - i * (uint32_t)L;
+                    si[hh] = i;
+                    sj[hh] = j;
                     const uint32_t iu = i == 0 ? L - 1 : i - 1, id = i == (uint32_t)L - 1 ? 0 : i + 1;
                     RingEntry en;
                     uint2 own = make_uint2(0u, 0u);
@@ -403,30 +407,29 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
                         if (REG) bits[at + RING] = own;
                     }
                 }
-            }
-            __syncwarp();
-            if (!REG) {
-                // relation codes of the new trials to the DEPTH trials before each
-                #pragma unroll 1
-                for (int r = 0; r < CHUNK / G; ++r) {
-                    const unsigned q = (unsigned)(2 * (c0 + cfill)) + (unsigned)(gl + r * G);
-                    const unsigned at = q & RMASK;
-                    const uint32_t b = ring[at].b, site = b >> 20;
-                    const uint32_t i = __umulhi(site, divL);
-                    const uint32_t j = site - i * (uint32_t)L;
-                    const uint32_t pos[5] = {j == 0 ? site + L - 1 : site - 1, site, j == (uint32_t)L - 1 ? site + 1 - L : site + 1,
-                                             i == 0 ? site + N - L : site - L, i == (uint32_t)L - 1 ? site + L - N : site + L};
-                    uint32_t rel = 0;
+                if (!REG) {
+                    // relation codes of the two trials to the DEPTH trials before each
+                    __syncwarp();
+                    uint32_t f[DEPTH + 1];          // sites of the trials before the second one, the nearest first
+                    f[0] = si[0] * (uint32_t)L + sj[0];
                     #pragma unroll
-                    for (int lag = 1; lag <= DEPTH; ++lag) {
-                        const uint32_t f = ring[(q - lag) & RMASK].b >> 20;
+                    for (int lag = 1; lag <= DEPTH; ++lag) f[lag] = ring[((unsigned)(2 * c) - lag) & RMASK].b >> 20;
+                    #pragma unroll
+                    for (int hh = 0; hh < 2; ++hh) {
+                        const uint32_t i = si[hh], j = sj[hh], site = i * (uint32_t)L + j;
+                        const uint32_t pos[5] = {j == 0 ? site + L - 1 : site - 1, site, j == (uint32_t)L - 1 ? site + 1 - L : site + 1,
+                                                 i == 0 ? site + N - L : site - L, i == (uint32_t)L - 1 ? site + L - N : site + L};
+                        uint32_t rel = site << 20;
                         #pragma unroll
-                        for (int k = 0; k < 5; ++k)
-                            if (f == pos[k]) rel |= 1u << (5 * (lag - 1) + k);
+                        for (int lag = 1; lag <= DEPTH; ++lag) {
+                            #pragma unroll
+                            for (int k = 0; k < 5; ++k)
+                                if (f[lag - hh] == pos[k]) rel |= 1u << (5 * (lag - 1) + k);
+                        }
+                        const unsigned at = (unsigned)(2 * c + hh) & RMASK;
+                        ring[at].b = rel;
+                        if (at < RING_TAIL) ring[at + RING].b = rel;
                     }
-                    rel |= site << 20;
-                    ring[at].b = rel;
-                    if (at < RING_TAIL) ring[at + RING].b = rel;
                 }
             }
             cfill += CHUNK / 2;
@@ -690,12 +693,18 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
     const int walkers_per_block = gpw * warps;
     const int blocks = (p.nwalk + walkers_per_block - 1) / walkers_per_block;
     const int threads = 32 * warps;
+    // Shared memory for the blocks an SM gets and no more: the rest is L1, which
+    // the tables live in.  The driver's choice goes by the blocks that could be
+    // resident, and may leave 28 KB of L1 (10,752 walkers at L = 32, 8 lanes: 4.3
+    // ms; 2.8 with 60 KB or more).
+    const size_t held = (smem + 1024) * (size_t)((p.sharing + 152ll * walkers_per_block - 1) / (152ll * walkers_per_block));
+    const int carve = (int)std::min<size_t>(100, (held * 100 + 228 * 1024 - 1) / (228 * 1024));
     auto go = [&](auto kern) -> cudaError_t {
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        return launch_next(kern, dim3(blocks), dim3(threads), smem, s, p, (unsigned)ntrials, (int)per);
+        return launch_next_with(carve, kern, dim3(blocks), dim3(threads), smem, s, p, (unsigned)ntrials, (int)per);
     };
     const int lat = p.lattice_reg ? (p.N <= 32 ? 1 : 2) : blocks_of(p.L).n > 1 ? 3 : 0;
     auto with = [&](auto staged, auto g, auto prec) -> cudaError_t {
