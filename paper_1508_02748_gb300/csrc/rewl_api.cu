@@ -280,18 +280,19 @@ int max_pairs_of(const Dims &d)
 // fixes stays.  Every choice gives the same chains.  Times are ms per 10^4
 // trials of every walker on a GB300.
 //   - Staged tables while all walkers fit on the GPU's shared memory at once:
-//     L = 8, 3 x 3 windows, staged against global: 36 walkers 0.43 / 0.57, 1350
-//     0.63 / 0.81; past that the staged walkers take turns: 1800 0.94 / 0.81.
-//   - Staged: 32 lanes up to one warp per SM sub-partition (450 walkers 0.43,
-//     16 lanes 0.49), then 16 (900: 0.53 against 0.49); more walkers make the
+//     L = 8, 3 x 3 windows, staged against global: 36 walkers 0.36 / 0.55, 1350
+//     0.60 / 0.81; past that the staged walkers take turns (1800: 0.97 with 16
+//     lanes, global 0.82).
+//   - Staged: 32 lanes up to two warps per SM sub-partition (900 walkers 0.47,
+//     16 lanes 0.49), then 16 (1350: 0.62 against 0.60); more walkers make the
 //     step's instructions count, fewer its depth.
-//   - Global: 32 lanes while that is at most 16 warps an SM (L = 32, 2048
-//     walkers: 1.05, 16 lanes 1.28; 2560: 1.47 against 1.37), 16 lanes while
-//     that is at most the 18 warps an SM that the registers allow (5120: 16
-//     lanes 1.72, 8 lanes 2.31), then 8 (8192: 2.91 against 2.53).
-//   - A lattice of N <= 64 in a register beside staged tables and with 8 lanes
-//     (1.50 against 1.69); with global tables and more lanes its longer chain
-//     costs more than its loads save (0.57 against 0.69 at 32).
+//   - Global: 32 lanes while that is at most the 18 warps an SM that the
+//     registers allow (L = 32, 2048 walkers 1.03, 16 lanes 1.19; 2560: 1.16 and
+//     1.27; 3072: 1.52 and 1.36), 16 lanes while that is (5120: 1.65, 8 lanes
+//     2.05; 6144: 2.34 and 2.16), then 8.
+//   - A lattice of N <= 64 in registers beside staged tables and with 8 lanes
+//     (0.83 against 0.98); with global tables and more lanes its longer chain
+//     costs more than its loads save (0.57 against 0.69 at 32 lanes).
 void choose_tiling(rewl_t *h, long long walkers)
 {
     constexpr long long kSMs = 152;
@@ -300,9 +301,9 @@ void choose_tiling(rewl_t *h, long long walkers)
     const rewl_config &c = h->cfg;
     const bool small = p.N <= 64 && p.wpr == 1 && c.lattice_mode != REWL_LATTICE_SHARED;
     const long long per_sm = (walkers + kSMs - 1) / kSMs;
-    const int staged_lanes = c.lanes_per_walker ? c.lanes_per_walker : walkers <= 4 * kSMs ? 32 : 16;
+    const int staged_lanes = c.lanes_per_walker ? c.lanes_per_walker : walkers <= 8 * kSMs ? 32 : 16;
     const int global_lanes = c.lanes_per_walker ? c.lanes_per_walker
-                           : walkers <= 16 * kSMs ? 32 : walkers <= 36 * kSMs ? 16 : 8;
+                           : walkers <= 18 * kSMs ? 32 : walkers <= 36 * kSMs ? 16 : 8;
     p.lattice_reg = small ? 1 : 0;
     const size_t gpw = (size_t)(32 / staged_lanes);
     const size_t block = tree_smem_per_warp(p, true, staged_lanes) * gpw + kPerBlock;

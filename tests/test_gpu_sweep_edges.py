@@ -70,8 +70,9 @@ def test_staged_narrow_rows(P, lattice):
 
 # either side of each line of the automatic tiling (staged or global tables,
 # 32, 16 or 8 lanes, lattice in a register or not), against the thread sampler
-@pytest.mark.parametrize("L,nE,nM,W", [(4, 1, 1, 608), (4, 1, 1, 609), (8, 3, 3, 185), (8, 3, 3, 186), (8, 3, 3, 271),
-                                       (6, 3, 2, 912), (6, 3, 2, 913), (12, 2, 1, 76), (12, 2, 1, 77)])
+@pytest.mark.parametrize("L,nE,nM,W", [(4, 1, 1, 608), (4, 1, 1, 609), (4, 2, 1, 608), (4, 2, 1, 609), (8, 3, 3, 185),
+                                       (8, 3, 3, 186), (8, 3, 3, 271), (8, 3, 3, 304), (8, 3, 3, 305), (6, 3, 2, 912),
+                                       (6, 3, 2, 913), (12, 2, 1, 76), (12, 2, 1, 77)])
 def test_automatic_tiling(P, L, nE, nM, W):
     kw = dict(L=L, n_win_E=nE, n_win_M=nM, walkers_per_window=W, seed=40 + L, exchange_interval=700)
     a, b = P.REWL(P.Config(**kw)), P.REWL(P.Config(sampler=P.SAMPLER_THREAD, **kw))
