@@ -507,6 +507,8 @@ __global__ void __launch_bounds__(256) k_flat(Params p)
     const int rank = SPLIT ? (int)cl.block_rank() : 0, parts = SPLIT ? (int)cl.num_blocks() : 1;
     const int w = (int)blockIdx.x / parts;
     if (!p.active[w / p.W]) return;            // (the whole cluster)
+    if constexpr (SPLIT) cg::cluster_group::barrier_arrive();   // waited for before the first block's memory is written:
+                                                                // it exists only once that block has started
     const int32_t *H = p.H + (size_t)w * p.tstride;
     long long cnt = 0, sum = 0;
     int mn = 0x7FFFFFFF;
@@ -534,9 +536,12 @@ __global__ void __launch_bounds__(256) k_flat(Params p)
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int k = 1; k < 8; ++k) { cnt += s_warp[k].cnt; sum += s_warp[k].sum; mn = min(mn, s_warp[k].mn); }
-        if constexpr (SPLIT) *cl.map_shared_rank(&s_block[rank], 0) = {cnt, sum, mn};
     }
-    if constexpr (SPLIT) cl.sync();
+    if constexpr (SPLIT) {
+        cg::cluster_group::barrier_wait();
+        if (threadIdx.x == 0) *cl.map_shared_rank(&s_block[rank], 0) = {cnt, sum, mn};
+        cl.sync();
+    }
     if (rank == 0 && threadIdx.x == 0) {
         for (int k = 1; k < parts; ++k) { cnt += s_block[k].cnt; sum += s_block[k].sum; mn = min(mn, s_block[k].mn); }
         const int flat = cnt > 0 && (long long)mn * cnt * 1000000ll >= p.flat_q * sum;
