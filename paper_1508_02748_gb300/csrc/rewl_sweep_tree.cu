@@ -274,9 +274,11 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
     const uint32_t divL = p.divL;
 
     // This lane's node of the tree.  Lane G-1 holds none: it never accepts and
-    // its move is 0.
-    const int dl = 31 - __clz(gl + 1);
+    // its move is 0; it goes along with the root's trial, which the ring always
+    // holds (the entry after the step's last trial may not be filled yet, and
+    // says which lattice words to read).
     const bool node = gl < G - 1;
+    const int dl = node ? 31 - __clz(gl + 1) : 0;
     const int hist = node ? gl + 1 - (1 << dl) : 0;
     const int spanp = node ? ((R.y - R.x) << 16) | (R.w - R.z) : (int)0xC0000000;
     // Lanes of the accepted trials of the history, the latest first (lane G-1
