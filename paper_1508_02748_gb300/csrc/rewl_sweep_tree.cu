@@ -74,7 +74,7 @@
 // shuffle).  Reading one bin a lane instead of two, the visit counts by three
 // comparisons, the leaf by shuffle instead of a mailbox, the trial read a step
 // ahead and near-ties looked at on the path alone took 266-302 instructions a
-// step to 145-150.  Sampling launches of 10^4 trials per walker, GB300, 2070
+// step to 149-157.  Sampling launches of 10^4 trials per walker, GB300, 2070
 // MHz, before -> after: L = 8 (36 walkers, 32 lanes, staged) 0.72 -> 0.35 ms; L
 // = 16 (256 walkers, 32 lanes) 0.95 -> 0.63 ms; L = 32 (2048 walkers, 32 lanes)
 // 1.64 -> 1.03 ms; L = 64 (3904 walkers, 16 lanes) 2.71 -> 1.56 ms.
