@@ -58,21 +58,45 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// Sums of exp(v - top) compare values by their upper words, which order like
-// them (an FP64 comparison occupies its pipe like an addition does): the top
-// needs only to be near the largest value, and a term is left out where it is
-// certainly LSE_FAR below.
-__device__ __forceinline__ int order_of(double v)
+// Sums of exp(v - top) find the top, the largest value, by integers (an FP64
+// comparison occupies its pipe like an addition does): the bits of a double,
+// the negative ones' flipped but for the sign, order like the value.  All 64 of
+// them count: a top that misses the largest value by a part in 2^20 lets exp
+// overflow from ln g = 2^30 on, and cuts all terms off below -2^26.
+__device__ __forceinline__ int order_of(double v)              // of the upper word alone
 {
     const int h = __double2hiint(v);
     return h ^ ((h >> 31) & 0x7FFFFFFF);
 }
 
 constexpr int ORDER_NONE = (int)0xFFF00000 ^ 0x7FFFFFFF;       // of -infinity
+constexpr long long KEY_NONE = (long long)ORDER_NONE * (1ll << 32) + 0xFFFFFFFFll;
 
-__device__ __forceinline__ double top_of(int order)
+__device__ __forceinline__ long long key_of(double v)
 {
-    return __hiloint2double(order ^ ((order >> 31) & 0x7FFFFFFF), 0);
+    const unsigned sign = (unsigned)(__double2hiint(v) >> 31);
+    return (long long)(((unsigned long long)(unsigned)order_of(v) << 32) | ((unsigned)__double2loint(v) ^ sign));
+}
+
+__device__ __forceinline__ double value_of(long long key)
+{
+    const int h = (int)(key >> 32);
+    return __hiloint2double(h ^ ((h >> 31) & 0x7FFFFFFF), (int)((unsigned)key ^ (unsigned)(h >> 31)));
+}
+
+__device__ __forceinline__ long long warp_max_key(long long k)
+{
+    const int h = (int)(k >> 32), m = __reduce_max_sync(0xFFFFFFFFu, h);
+    const unsigned l = __reduce_max_sync(0xFFFFFFFFu, h == m ? (unsigned)k : 0u);
+    return (long long)(((unsigned long long)(unsigned)m << 32) | l);
+}
+
+// The upper words tell which terms are certainly LSE_FAR below the top, `far`
+// the order of top - LSE_FAR; what is not a number counts as a term (the
+// negative ones order below -infinity).
+__device__ __forceinline__ bool counts(double v, int far)
+{
+    return (unsigned)order_of(v) - (unsigned)ORDER_NONE >= (unsigned)far - (unsigned)ORDER_NONE;
 }
 
 // ln sum_i exp(v[i]) over the finite v[0..n) by one warp: the top, then the
@@ -80,16 +104,16 @@ __device__ __forceinline__ double top_of(int order)
 __device__ __forceinline__ double lse_warp(const double *v, int n)
 {
     const int lane = threadIdx.x & 31;
-    int mo = ORDER_NONE;
-    for (int i = lane; i < n; i += 32) mo = max(mo, order_of(v[i]));
-    mo = __reduce_max_sync(0xFFFFFFFFu, mo);
-    if (mo == ORDER_NONE) return -INFINITY;
-    const double top = top_of(mo);
+    long long key = KEY_NONE;
+    for (int i = lane; i < n; i += 32) key = max(key, key_of(v[i]));
+    key = warp_max_key(key);
+    if (key == KEY_NONE) return -INFINITY;
+    const double top = value_of(key);
     const int far = order_of(top - LSE_FAR);
     double acc = 0.0;
     for (int i = lane; i < n; i += 32) {
         const double x = v[i];
-        if (order_of(x) >= far) acc += exp(x - top);
+        if (counts(x, far)) acc += exp(x - top);
     }
     return top + log(warp_sum(acc));
 }
@@ -504,23 +528,23 @@ __global__ void __launch_bounds__(ROW_COLS * ROW_ES) k_marg_row(Params p, JoinSc
             for (int e = from + ex; e < to; e += ROW_ES) f(col[(size_t)(e - e0) * p.wM] + c);
         }
     };
-    __shared__ int s_top[ROW_ES][ROW_COLS];
-    int mo = ORDER_NONE;
-    each([&](double v) { mo = max(mo, order_of(v)); });
-    s_top[ex][cx] = mo;
+    __shared__ long long s_top[ROW_ES][ROW_COLS];
+    long long key = KEY_NONE;
+    each([&](double v) { key = max(key, key_of(v)); });
+    s_top[ex][cx] = key;
     __syncthreads();
-    for (int k = 0; k < ROW_ES; ++k) mo = max(mo, s_top[k][cx]);
-    const double top = top_of(mo);
+    for (int k = 0; k < ROW_ES; ++k) key = max(key, s_top[k][cx]);
+    const double top = value_of(key);
     double acc = 0.0;
-    if (mo != ORDER_NONE) {
+    if (key != KEY_NONE) {
         const int far = order_of(top - LSE_FAR);
-        each([&](double v) { if (order_of(v) >= far) acc += exp(v - top); });
+        each([&](double v) { if (counts(v, far)) acc += exp(v - top); });
     }
     s_part[ex][cx] = acc;
     __syncthreads();
     if (ex == 0 && m < B) {
         for (int k = 1; k < ROW_ES; ++k) acc += s_part[k][cx];
-        j.F[(size_t)b * B + m] = mo == ORDER_NONE ? -INFINITY : top + log(acc);
+        j.F[(size_t)b * B + m] = key == KEY_NONE ? -INFINITY : top + log(acc);
     }
 }
 
@@ -575,15 +599,15 @@ __global__ void __launch_bounds__(MATCH_THREADS) k_match_m(Params p, JoinScratch
     }
 }
 
-// 3c. Assemble the joined table; each block leaves the order of the largest
-// value of its part in red[].
-constexpr int RED_BLOCKS = 512;     // red[]: 512 maxima (their order), then from entry 512 on the sums
+// 3c. Assemble the joined table; each block leaves the key of the largest value
+// of its part in red[].
+constexpr int RED_BLOCKS = 512;     // red[]: 512 maxima (their keys), then from entry 512 on the sums
 
 __global__ void __launch_bounds__(256) k_assemble(Params p, JoinScratch j)
 {
     after_previous();
     const int B = p.N + 1;
-    int mo = ORDER_NONE;
+    long long key = KEY_NONE;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < (size_t)B * B; idx += (size_t)gridDim.x * blockDim.x) {
         const int e = (int)(idx / B), m = (int)(idx % B);
         double v = -INFINITY;
@@ -596,44 +620,44 @@ __global__ void __launch_bounds__(256) k_assemble(Params p, JoinScratch j)
             }
         }
         j.J[idx] = v;
-        mo = max(mo, order_of(v));
+        key = max(key, key_of(v));
     }
-    mo = __reduce_max_sync(0xFFFFFFFFu, mo);
-    __shared__ int s[8];
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = mo;
+    key = warp_max_key(key);
+    __shared__ long long s[8];
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = key;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < 8; ++k) mo = max(mo, s[k]);
-        reinterpret_cast<int *>(j.red)[blockIdx.x] = mo;
+        for (int k = 1; k < 8; ++k) key = max(key, s[k]);
+        reinterpret_cast<long long *>(j.red)[blockIdx.x] = key;
     }
 }
 
 // 4. Normalisation: sums of exp(v - max) by blocks, then the shift that makes
 // sum g = 2^N.  Each block folds the blocks' maxima (sums) itself, all in the
 // same order, instead of waiting for a kernel that does.
-__device__ __forceinline__ int fold_max(const double *red, int n)
+__device__ __forceinline__ long long fold_max(const double *red, int n)
 {
-    __shared__ int s_m[8];
-    int mo = ORDER_NONE;
-    for (int k = threadIdx.x; k < n; k += 256) mo = max(mo, reinterpret_cast<const int *>(red)[k]);
-    mo = __reduce_max_sync(0xFFFFFFFFu, mo);
-    if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = mo;
+    __shared__ long long s_m[8];
+    long long key = KEY_NONE;
+    for (int k = threadIdx.x; k < n; k += 256) key = max(key, reinterpret_cast<const long long *>(red)[k]);
+    key = warp_max_key(key);
+    if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = key;
     __syncthreads();
-    for (int k = 0; k < 8; ++k) mo = max(mo, s_m[k]);
-    return mo;
+    for (int k = 0; k < 8; ++k) key = max(key, s_m[k]);
+    return key;
 }
 
 __global__ void __launch_bounds__(256) k_red_sumexp(const double *v, size_t n, double *red, int nblk)
 {
     after_previous();
-    const int mo = fold_max(red, nblk);
-    const double top = top_of(mo);
+    const long long key = fold_max(red, nblk);
+    const double top = value_of(key);
     double acc = 0.0;
-    if (mo != ORDER_NONE) {
+    if (key != KEY_NONE) {
         const int far = order_of(top - LSE_FAR);
         for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
             const double x = v[i];
-            if (order_of(x) >= far) acc += exp(x - top);
+            if (counts(x, far)) acc += exp(x - top);
         }
     }
     acc = warp_sum(acc);
@@ -649,7 +673,7 @@ __global__ void __launch_bounds__(256) k_red_sumexp(const double *v, size_t n, d
 __global__ void __launch_bounds__(256) k_normalise(double *v, size_t n, const double *red, int nblk, int N)
 {
     after_previous();
-    const double top = top_of(fold_max(red, nblk));
+    const double top = value_of(fold_max(red, nblk));
     double acc = 0.0;
     for (int k = threadIdx.x; k < nblk; k += 256) acc += red[RED_BLOCKS + k];
     acc = warp_sum(acc);
