@@ -1,5 +1,7 @@
 """The join over the whole range of what it takes: ln g of large magnitude
 against the oracle, and grids of more windows than one grid axis has blocks."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -47,3 +49,37 @@ def test_join_of_large_tables(P, offset, nE, nM):
             fin = np.isfinite(Jo)
             assert np.array_equal(np.isfinite(Jg), fin)
             np.testing.assert_allclose(Jg[fin], Jo[fin], rtol=0, atol=tol)
+
+
+def test_join_of_more_windows_than_a_grid_axis(P):
+    """257 x 257 windows of 2 x 2 bins cut out of one table, each with an offset
+    of its own: joined again, the table comes back up to a constant.  It falls
+    off by 50 a bin beside a ridge that all windows of an m range hold with its
+    neighbours, so that rows of different length agree on their marginals."""
+    import torch
+    L, n = 16, 257
+    cfg = P.Config(L=L, n_win_E=n, n_win_M=n, overlap_E=0.5, overlap_M=0.5)
+    lo = (2 * np.arange(n) * (n - 2) + n - 1) // (2 * (n - 1))              # window starts, rounded half up
+    can = np.array([[oracle.lib().orc_bin_possible(L, e, m) for m in range(n)] for e in range(n)]) != 0
+    e = np.arange(n)[:, None]
+    ridge = np.array([np.flatnonzero(can[:, m]).mean().round() for m in range(n)])
+    G = -50.0 * np.abs(e - ridge[None, :])
+    rng = np.random.default_rng(4)
+    two = np.arange(2)
+    rows, cols = lo[None, :, None, None] + two[:, None], lo[:, None, None, None] + two[None, :]
+    tab = G[rows, cols] + np.round(rng.uniform(0, 900, (n, n, 1, 1)) * 64) / 64
+    d = torch.from_numpy(np.ascontiguousarray(tab).ravel()).cuda()
+    H = torch.ones(d.numel(), dtype=torch.int32, device="cuda")
+    out = torch.empty(n, n, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    lib, c = P.load_library(), cfg.to_c()
+    rc = lib.rewl_join_noalloc(ctypes.byref(c), d.data_ptr(), H.data_ptr(), out.data_ptr(), None)
+    assert rc == 0, lib.rewl_noalloc_last_error()
+    J = out.cpu().numpy()
+    fin = np.isfinite(J)
+    assert fin[can].all()
+    diff = (J - G)[fin]
+    # 512 matching points, at each two marginals, their difference and a shift, of at most 2^14 in magnitude
+    assert np.ptp(diff) < 2 * 512 * 4 * 2.0**-53 * 2**14
+    top = J[fin].max()
+    np.testing.assert_allclose(top + np.log(np.exp(J[fin] - top).sum()), L * L * np.log(2.0), rtol=0, atol=1e-9)
