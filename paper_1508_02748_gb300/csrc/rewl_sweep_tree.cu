@@ -169,6 +169,16 @@ __device__ __forceinline__ int exact_accept(const typename TB::Elem *gb, unsigne
     return log(unit_open_d((q & 1ull) ? x.w : x.y)) < delta ? 1 : 0;
 }
 
+// Four bytes into shared memory; no register waits for them, so that one warp
+// has a whole window under way.
+__device__ __forceinline__ void async4(void *to, const void *from)
+{
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(to);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(from) : "memory");
+}
+
+__device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <int G>
 struct TreeShape {
     static constexpr int DEPTH = G == 32 ? 4 : G == 16 ? 3 : 2;
@@ -226,7 +236,38 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
     const int ld = staged_ld(wM);
     const int nstaged = (p.wE + 4) * ld;
     int2 *tab = reinterpret_cast<int2 *>(base + RING_BYTES + (REG ? BITS_BYTES : ((nlat + G) * 4 + 15) & ~15));
-    if constexpr (SMT) {
+    // Staging in and out of a window by one warp: the entries come by copies
+    // that no register waits for, their addresses by a walk through the rows
+    // (loads, stores and a division an entry before: 3.4 ns a bin in and out, 1.4
+    // so; L = 8's 64 cycles 23.2 -> 22.4 ms).  Windows of at most 26 x 26 bins
+    // (N <= 32) keep the short form: they have little to stage, and the step
+    // compiled with the walk took 2% longer there.
+    constexpr bool WALK = SMT && LAT != 1;
+    auto each_bin = [&](auto f) {                   // f(bin, its entry), every G-th one
+        const int by = G / wM;                      // rows that G bins are on
+        int m = gl % wM, k = (gl / wM + 2) * ld + m;
+        #pragma unroll 4
+        for (int b = gl; b < p.T; b += G) {
+            f(b, k);
+            m += G - by * wM;
+            k += G + by * (ld - wM);
+            if (m >= wM) {
+                m -= wM;
+                k += ld - wM;
+            }
+        }
+    };
+    if constexpr (WALK) {
+        each_bin([&](int b, int k) {
+            async4(&tab[k].x, gS + b);
+            async4(&tab[k].y, gH + b);
+        });
+        for (int k = gl; k < 2 * ld; k += G) tab[k] = tab[nstaged - 1 - k] = make_int2(0, -1);
+        for (int e = 2 + gl; e < p.wE + 2; e += G)
+            for (int m = wM; m < ld; ++m) tab[e * ld + m] = make_int2(0, -1);
+        async_wait();
+        each_bin([&](int, int k) { atomicMax(&tab[k].y, 0); });
+    } else if constexpr (SMT) {
         #pragma unroll 4
         for (int k = gl; k < nstaged; k += G) {
             const int e = k / ld - 2, m = k - (e + 2) * ld;
@@ -629,7 +670,12 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
     if (__any_sync(FULL, err < 0) && lane == 0) atomicOr(&p.st->error, ERR_OVERFLOW);
     __syncwarp();
     if (idle) return;
-    if constexpr (SMT) {
+    if constexpr (WALK) {
+        each_bin([&](int b, int k) {
+            const int h = tab[k].y;
+            if (h > 0) gH[b] = h;
+        });
+    } else if constexpr (SMT) {
         for (int k = gl + 2 * ld; k < nstaged - 2 * ld; k += G) {
             const int e = k / ld - 2, m = k - (e + 2) * ld, h = tab[k].y;
             if (m < wM && h > 0) gH[e * wM + m] = h;

@@ -1,0 +1,33 @@
+"""The warp sampler with its tables staged against the same run with them in
+global memory, bit for bit: windows narrower and wider than a walker's lanes."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1508_02748_gb300 as P
+    from paper_1508_02748_gb300 import build
+    build.build()
+    return P
+
+
+# rows of 7 to 145 bins, windows of 16 to 145 rows, every form of the lattice
+# (N <= 32, N <= 64, one block a row, several), launches of a few trials
+@pytest.mark.parametrize("L,nE,nM,W,lanes", [(5, 1, 5, 3, 16), (6, 1, 12, 3, 32), (6, 1, 12, 3, 8), (6, 1, 19, 2, 16), (7, 10, 1, 3, 16),
+                                             (8, 2, 9, 3, 8), (8, 13, 2, 2, 32), (9, 1, 6, 3, 32), (10, 4, 4, 3, 16), (12, 1, 1, 3, 32),
+                                             (31, 24, 24, 1, 32)])
+def test_staged_equals_global(P, L, nE, nM, W, lanes):
+    kw = dict(L=L, n_win_E=nE, n_win_M=nM, overlap_E=0.75, overlap_M=0.75, walkers_per_window=W, seed=70 + L, lanes_per_walker=lanes,
+              drive_budget=10**9)
+    a, b = (P.REWL(P.Config(table_mode=t, **kw)) for t in (P.TABLES_STAGED, P.TABLES_GLOBAL))
+    for n in (1, 7, 900):
+        a.sweep(n)
+        b.sweep(n)
+        for x, y in zip(a.walkers() + a.tables(), b.walkers() + b.tables()):
+            np.testing.assert_array_equal(x, y)
