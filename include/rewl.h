@@ -67,7 +67,7 @@ extern "C" {
 /* Where the warp sampler keeps a walker's screen and visit counts during a
  * launch (rewl_config.table_mode); every choice gives the same trajectory. */
 #define REWL_TABLES_AUTO 0      /* staged when the windows of all walkers fit in the GPU's shared memory
-                                   at once, else global */
+                                   at once and a launch has the trials to pay for it, else global */
 #define REWL_TABLES_GLOBAL 1    /* global memory (L1-cached) */
 #define REWL_TABLES_STAGED 2    /* all of the walker's bins in shared memory for the launch (REWL_E_CUDA
                                    at launch when they do not fit) */

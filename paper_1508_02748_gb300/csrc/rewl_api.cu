@@ -275,14 +275,19 @@ int max_pairs_of(const Dims &d)
     return best;
 }
 
-// How the warp sampler maps a run onto the GPU when `walkers` walkers (its
-// own, or those of all runs of a batch) share it; what the configuration
-// fixes stays.  Every choice gives the same chains.  Times are ms per 10^4
-// trials of every walker on a GB300.
+// How the warp sampler maps launches of `trials` trials onto the GPU when
+// `walkers` walkers (the run's own, or those of all runs of a batch) share it;
+// what the configuration fixes stays.  Every choice gives the same chains.
+// Times are ms per 10^4 trials of every walker on a GB300.
 //   - Staged tables while all walkers fit on the GPU's shared memory at once:
 //     L = 8, 3 x 3 windows, staged against global: 36 walkers 0.36 / 0.55, 1350
 //     0.60 / 0.81; past that the staged walkers take turns (1800: 0.97 with 16
 //     lanes, global 0.82).
+//   - And while the launch pays for the staging, some 1.4 ns a bin against 10
+//     ns a trial (20 with a register lattice): from a trial for 12 (16) bins on.
+//     One window, us a cycle staged / global: L = 12 (21,025 bins) 48 / 21 at
+//     100 trials, 85 / 74 at 1000, 172 / 185 at 3000; L = 10 (10,201) 39 / 30 at
+//     300, 68 / 71 at 1000; L = 8 (4225) 21 / 17 at 100, 27 / 30 at 300.
 //   - Staged: 32 lanes up to two warps per SM sub-partition (900 walkers 0.47,
 //     16 lanes 0.49), then 16 (1350: 0.62 against 0.60); more walkers make the
 //     step's instructions count, fewer its depth.
@@ -293,12 +298,10 @@ int max_pairs_of(const Dims &d)
 //   - A lattice of N <= 64 in registers beside staged tables and with 8 lanes
 //     (0.83 against 0.98); with global tables and more lanes its longer chain
 //     costs more than its loads save (0.57 against 0.69 at 32 lanes).
-void choose_tiling(rewl_t *h, long long walkers)
+void choose_tiling(Params &p, const rewl_config &c, long long walkers, uint64_t trials)
 {
     constexpr long long kSMs = 152;
     constexpr size_t kSmem = 227 * 1024, kPerBlock = 1024;
-    Params &p = h->p;
-    const rewl_config &c = h->cfg;
     const bool small = p.N <= 64 && p.wpr == 1 && c.lattice_mode != REWL_LATTICE_SHARED;
     const long long per_sm = (walkers + kSMs - 1) / kSMs;
     const int staged_lanes = c.lanes_per_walker ? c.lanes_per_walker : walkers <= 8 * kSMs ? 32 : 16;
@@ -310,7 +313,7 @@ void choose_tiling(rewl_t *h, long long walkers)
     const size_t blocks = (size_t)((per_sm + (long long)gpw - 1) / (long long)gpw);
     if (p.sampler != REWL_SAMPLER_WARP) p.smt = 0;
     else if (c.table_mode != REWL_TABLES_AUTO) p.smt = c.table_mode == REWL_TABLES_STAGED;
-    else p.smt = block * (blocks ? blocks : 1) <= kSmem + kPerBlock;
+    else p.smt = block * (blocks ? blocks : 1) <= kSmem + kPerBlock && trials >= (uint64_t)(p.T / (small ? 16 : 12));
     p.group = p.smt ? staged_lanes : global_lanes;
     p.sharing = walkers;
     if (c.lattice_mode == REWL_LATTICE_AUTO && !p.smt && p.group != 8) p.lattice_reg = 0;
@@ -562,7 +565,7 @@ int create_impl(const rewl_config *cfg, const uint8_t *host_init_spins, void *d_
             n_active += any ? 1 : 0;
         }
     p.n_active_walkers = n_active * d.W;
-    choose_tiling(h, p.n_active_walkers);
+    choose_tiling(p, h->cfg, p.n_active_walkers, h->cfg.exchange_interval);
     h->first_active = -1;
     for (int win = 0; win < d.nwin && h->first_active < 0; ++win)
         if (active[win]) h->first_active = win * d.W;
@@ -852,7 +855,9 @@ extern "C" int rewl_run_iteration(rewl_t *h, uint64_t max_cycles, rewl_status *s
 extern "C" int rewl_sweep(rewl_t *h, uint64_t n_trials)
 {
     if (!h) return REWL_E_INVALID;
-    CK(h, launch_sweep(h->p, n_trials, h->wpb, h->stream));
+    Params p = h->p;
+    choose_tiling(p, h->cfg, p.n_active_walkers, n_trials);
+    CK(h, launch_sweep(p, n_trials, h->wpb, h->stream));
     DevState ds;
     return read_state(h, &ds);
 }
@@ -1243,7 +1248,7 @@ extern "C" int rewl_batch_create(rewl_t *const *runs, int n, void *stream, rewl_
         cudaStream_t own = h->stream;
         const Params alone = h->p;
         h->stream = b->streams[i];
-        choose_tiling(h, walkers);
+        choose_tiling(h->p, h->cfg, walkers, h->cfg.exchange_interval);
         qe = cudaStreamWaitEvent(h->stream, b->events[n], 0);
         const unsigned long long ce = (unsigned long long)h->cfg.check_every;
         for (unsigned long long c = 0; c < b->k && qe == cudaSuccess; ++c)

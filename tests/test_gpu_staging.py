@@ -31,3 +31,22 @@ def test_staged_equals_global(P, L, nE, nM, W, lanes):
         b.sweep(n)
         for x, y in zip(a.walkers() + a.tables(), b.walkers() + b.tables()):
             np.testing.assert_array_equal(x, y)
+
+
+# The automatic placement with launches of few trials: staging a window would
+# take longer than sampling it (at 100 trials 4.5 and 2.2 times as long as a
+# cycle from global memory, which the limit of 1.5 tells apart).
+@pytest.mark.parametrize("L,W", [(12, 1), (12, 152), (10, 4)])
+def test_short_launches_do_not_stage(P, L, W):
+    import time
+    us = []
+    for mode in (P.TABLES_AUTO, P.TABLES_GLOBAL):
+        r = P.REWL(P.Config(L=L, walkers_per_window=W, seed=3, exchange_interval=100, lnf_final=1e-8, table_mode=mode))
+        r.run_cycles(64)
+        best = float("inf")
+        for _ in range(10):
+            t = time.perf_counter()
+            r.run_cycles(64)
+            best = min(best, time.perf_counter() - t)
+        us.append(best / 64 * 1e6)
+    assert us[0] < 1.5 * us[1], us
