@@ -731,8 +731,9 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
     const size_t per = tree_smem_per_warp(p, smt, group);
     // one warp a block: blocks of several warps leave when their last walker
     // does (16 lanes, L = 16: 0.90 ms at 1 warp, 1.00 at 4; 32 lanes: the same);
-    // and many walkers' blocks of four 8-lane groups do not all become resident
-    // (10,752 walkers at L = 32: 4.28 ms, 2.77 at two warps)
+    // with four 8-lane groups a warp two (L = 32, shared memory set aside as
+    // below: 9600 walkers 2.61 ms at 1 warp, 2.50 at 2 and 4; 10,752: 2.97, 2.72,
+    // 2.74; 11,520: 4.23, 3.03, 2.81)
     if (warps <= 0) warps = group == 8 ? 2 : 1;
     // no more warps per block than the shared memory of one block holds
     while (warps > 1 && per * (size_t)gpw * warps > max_smem) --warps;
@@ -744,15 +745,23 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
     // Shared memory for the blocks an SM gets and no more: the rest is L1, which
     // the tables live in.  The driver's choice goes by the blocks that could be
     // resident, and may leave 28 KB of L1 (10,752 walkers at L = 32, 8 lanes: 4.3
-    // ms; 2.8 with 60 KB or more).
-    const size_t held = (smem + 1024) * (size_t)((p.sharing + 152ll * walkers_per_block - 1) / (152ll * walkers_per_block));
-    const int carve = (int)std::min<size_t>(100, (held * 100 + 228 * 1024 - 1) / (228 * 1024));
+    // ms; 2.8 with 60 KB or more).  Past some 11,000 walkers their blocks take
+    // turns, and only those that an SM holds at once count (12,288 walkers 5.6 ->
+    // 3.7 ms, 16,384 7.4 -> 4.9, 24,576 9.9 -> 6.4).
+    const long long share = (p.sharing + 152ll * walkers_per_block - 1) / (152ll * walkers_per_block);
     auto go = [&](auto kern) -> cudaError_t {
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
+        cudaError_t e = cudaSuccess;
+        if (smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        long long held = share;
+        if (e == cudaSuccess && share * warps > 16) {
+            int fit = 0;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, threads, smem);
+            held = std::min<long long>(share, std::max(fit, 1));
         }
-        return launch_next_with(carve, kern, dim3(blocks), dim3(threads), smem, s, p, (unsigned)ntrials, (int)per);
+        if (e != cudaSuccess) return e;
+        const long long carve = ((long long)(smem + 1024) * held * 100 + 228 * 1024 - 1) / (228 * 1024);
+        return launch_next_with((int)std::min<long long>(100, carve), kern, dim3(blocks), dim3(threads), smem, s, p,
+                                (unsigned)ntrials, (int)per);
     };
     const int lat = p.lattice_reg ? (p.N <= 32 ? 1 : 2) : blocks_of(p.L).n > 1 ? 3 : 0;
     auto with = [&](auto staged, auto g, auto prec) -> cudaError_t {
