@@ -17,6 +17,76 @@
 
 using namespace rewl;
 
+namespace {
+
+// Pinned host memory for the small results of a call (state, matching points):
+// copies into it are queued behind the work and share one wait, where a copy
+// into pageable memory waits by itself.  A handle holds one block from creation
+// to destruction, after which it is kept for the next handles: freeing pinned
+// memory waits for all of the device's work (9.7 ms beside a kernel of 10 ms).
+// There are at most kPinMost blocks (4 MB), and a handle beyond them copies its
+// results one by one.  A block is used again only in the context that it was
+// made in (a reset of the device ends that one and frees the memory).
+constexpr size_t kPinBytes = 16 * 1024;
+constexpr int kPinMost = 256;
+
+struct Pin {
+    unsigned char *at;               // null: none
+    unsigned long long context;
+};
+
+std::mutex g_pin_mu;
+Pin g_pin_free[kPinMost];
+int g_pin_n = 0, g_pin_made = 0;
+
+// Number of the calling thread's context, which no other one ever gets; 0 if it cannot be told.
+unsigned long long context_number()
+{
+    static int (*const get_id)(void *, unsigned long long *) = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) != cudaSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<int (*)(void *, unsigned long long *)>(f);
+    }();
+    unsigned long long id = 0;
+    return get_id && get_id(nullptr, &id) == 0 ? id : 0;
+}
+
+Pin pin_take()
+{
+    const unsigned long long context = context_number();
+    if (context == 0) return {};
+    {
+        std::lock_guard<std::mutex> lk(g_pin_mu);
+        for (int i = g_pin_n - 1; i >= 0; --i)
+            if (g_pin_free[i].context == context) {
+                const Pin b = g_pin_free[i];
+                g_pin_free[i] = g_pin_free[--g_pin_n];
+                return b;
+            }
+        if (g_pin_made == kPinMost) return {};
+        ++g_pin_made;
+    }
+    void *b = nullptr;
+    if (cudaHostAlloc(&b, kPinBytes, cudaHostAllocPortable) == cudaSuccess) return {(unsigned char *)b, context};
+    cudaGetLastError();
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    --g_pin_made;
+    return {};
+}
+
+void pin_give(Pin b)
+{
+    if (!b.at) return;
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    g_pin_free[g_pin_n++] = b;
+}
+
+}  // namespace
+
 struct rewl_s {
     rewl_config cfg;
     Params p;
@@ -38,47 +108,10 @@ struct rewl_s {
     cudaStream_t plain_s[REWL_PLAIN_STREAMS];
     cudaEvent_t plain_ev[REWL_PLAIN_STREAMS + 1];
     bool plain_ok;
-    unsigned char *pin;              // kPinBytes of pinned host memory for small results, null if none was to be had
+    Pin pin;                         // kPinBytes of pinned host memory for small results
 };
 
 namespace {
-
-// Pinned host memory for the small results of a call (state, matching points):
-// copies into it are queued behind the work and share one wait, where a copy
-// into pageable memory waits by itself.  A handle holds one block from creation
-// to destruction; up to kPinKept returned blocks are kept for the next handles.
-constexpr size_t kPinBytes = 16 * 1024;
-constexpr int kPinKept = 32;
-std::mutex g_pin_mu;
-unsigned char *g_pin_free[kPinKept];
-int g_pin_n = 0;
-
-unsigned char *pin_take()
-{
-    {
-        std::lock_guard<std::mutex> lk(g_pin_mu);
-        if (g_pin_n > 0) return g_pin_free[--g_pin_n];
-    }
-    void *b = nullptr;
-    if (cudaHostAlloc(&b, kPinBytes, cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();          // (then results are copied one by one)
-        return nullptr;
-    }
-    return (unsigned char *)b;
-}
-
-void pin_give(unsigned char *b)
-{
-    if (!b) return;
-    {
-        std::lock_guard<std::mutex> lk(g_pin_mu);
-        if (g_pin_n < kPinKept) {
-            g_pin_free[g_pin_n++] = b;
-            return;
-        }
-    }
-    cudaFreeHost(b);
-}
 
 const char *g_noerr = "";
 char g_create_err[512];
@@ -339,8 +372,8 @@ struct Fetch {
     bool add(void *to, const void *dev, size_t bytes)
     {
         const size_t at = (used + 15) & ~(size_t)15;
-        if (!h->pin || n == 4 || at + bytes > kPinBytes || at + bytes < bytes) return false;
-        if (err == cudaSuccess) err = cudaMemcpyAsync(h->pin + at, dev, bytes, cudaMemcpyDeviceToHost, h->stream);
+        if (!h->pin.at || n == 4 || at + bytes > kPinBytes || at + bytes < bytes) return false;
+        if (err == cudaSuccess) err = cudaMemcpyAsync(h->pin.at + at, dev, bytes, cudaMemcpyDeviceToHost, h->stream);
         part[n++] = {to, at, bytes};
         used = at + bytes;
         return true;
@@ -353,12 +386,13 @@ struct Fetch {
     }
     cudaError_t wait()
     {
-        if (err == cudaSuccess) err = cudaStreamSynchronize(h->stream);
+        const cudaError_t e = cudaStreamSynchronize(h->stream);   // (also where a copy after the first was refused)
+        if (err == cudaSuccess) err = e;
         return err;
     }
     void give(int from = 0)
     {
-        for (int i = from; i < n; ++i) std::memcpy(part[i].to, h->pin + part[i].at, part[i].bytes);
+        for (int i = from; i < n; ++i) std::memcpy(part[i].to, h->pin.at + part[i].at, part[i].bytes);
     }
 };
 
@@ -491,7 +525,6 @@ int create_impl(const rewl_config *cfg, const uint8_t *host_init_spins, void *d_
     h->host_cycle = 0;
     h->wpb = cfg->walkers_per_block;
     h->graph_ok = false;
-    h->pin = pin_take();
     h->max_pairs = max_pairs_of(d);
 
     char *base = (char *)d_workspace;
@@ -586,6 +619,7 @@ int create_impl(const rewl_config *cfg, const uint8_t *host_init_spins, void *d_
         }                                                                                      \
     } while (0)
     CKB(cudaMemcpyAsync(p.st, &ds, sizeof(ds), cudaMemcpyHostToDevice, h->stream));
+    h->pin = pin_take();                 // (the thread has its context now)
     CKB(cudaMemcpyAsync((void *)p.rect, rect.data(), sizeof(int4) * d.nwin, cudaMemcpyHostToDevice, h->stream));
     CKB(cudaMemcpyAsync((void *)p.active, active.data(), sizeof(int32_t) * d.nwin, cudaMemcpyHostToDevice, h->stream));
     // Tables: ln g = 0, H = -1 (never visited).
@@ -1074,7 +1108,7 @@ extern "C" int rewl_get_lng(rewl_t *h, int what, double *host_out, size_t capaci
     const bool em = host_ematch && f.add(host_ematch, h->j.ematch, em_bytes);
     const bool mm = host_mmatch && f.add(host_mmatch, h->j.mmatch, mm_bytes);
     CK(h, f.wait());
-    if (states) std::memcpy(&ds, h->pin, sizeof(DevState));
+    if (states) std::memcpy(&ds, h->pin.at, sizeof(DevState));
     if (ds.error & ERR_OVERFLOW) return fail(h, REWL_E_OVERFLOW, "histogram entry above INT32_MAX");
     if (ds.join_error) return fail(h, REWL_E_JOIN, "join failed (code %d): adjacent pieces share no visited bins", ds.join_error);
     f.give(states);
