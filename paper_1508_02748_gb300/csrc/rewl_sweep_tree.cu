@@ -742,12 +742,16 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
     const int walkers_per_block = gpw * warps;
     const int blocks = (p.nwalk + walkers_per_block - 1) / walkers_per_block;
     const int threads = 32 * warps;
-    // Shared memory for the blocks an SM gets and no more: the rest is L1, which
-    // the tables live in.  The driver's choice goes by the blocks that could be
+    // Shared memory for the blocks an SM gets and little more: the rest is L1,
+    // which the tables live in.  The driver's choice goes by the blocks that could be
     // resident, and may leave 28 KB of L1 (10,752 walkers at L = 32, 8 lanes: 4.3
     // ms; 2.8 with 60 KB or more).  Past some 11,000 walkers their blocks take
     // turns, and only those that an SM holds at once count (12,288 walkers 5.6 ->
-    // 3.7 ms, 16,384 7.4 -> 4.9, 24,576 9.9 -> 6.4).
+    // 3.7 ms, 16,384 7.4 -> 4.9, 24,576 9.9 -> 6.4).  Other runs' blocks find a
+    // place beside a small run's only within its carve-out: 64 KB are 14 of their
+    // 32-lane warps (8 runs of 128 walkers at L = 16, each on its own stream: 2.11
+    // ms a cycle without, 0.79 so, one alone 0.61), and staged walkers, which need
+    // no L1, leave them all of it (32 runs of 36 at L = 8: 2.53 and 0.59).
     const long long share = (p.sharing + 152ll * walkers_per_block - 1) / (152ll * walkers_per_block);
     auto go = [&](auto kern) -> cudaError_t {
         cudaError_t e = cudaSuccess;
@@ -759,8 +763,9 @@ cudaError_t launch_sweep_tree(const Params &p, uint64_t ntrials, int group, int 
             held = std::min<long long>(share, std::max(fit, 1));
         }
         if (e != cudaSuccess) return e;
-        const long long carve = ((long long)(smem + 1024) * held * 100 + 228 * 1024 - 1) / (228 * 1024);
-        return launch_next_with((int)std::min<long long>(100, carve), kern, dim3(blocks), dim3(threads), smem, s, p,
+        const long long all = 228 * 1024;
+        const long long room = smt ? all : std::max<long long>((long long)(smem + 1024) * held, 64 * 1024);
+        return launch_next_with((int)std::min<long long>(100, (room * 100 + all - 1) / all), kern, dim3(blocks), dim3(threads), smem, s, p,
                                 (unsigned)ntrials, (int)per);
     };
     const int lat = p.lattice_reg ? (p.N <= 32 ? 1 : 2) : blocks_of(p.L).n > 1 ? 3 : 0;
