@@ -183,8 +183,31 @@ cudaError_t launch_drive(const Params &p, int32_t *d_fail, cudaStream_t s)
 // REG: the lattice (N <= 64, bit i*L + j) is one 64-bit register; otherwise
 // it lives in shared memory, word q of row r of thread t at
 // sm[(r * wpr + q) * nb + t], so the lanes of a warp never share a bank.
+//
+// ThreadParams: what it reads of Params, in an order of its own.  A lone thread
+// is a chain of latencies, and the generator's keys and the lattice's divisor,
+// read again in every trial, come in one piece where they lie on a 16-byte
+// boundary (off it, as in Params, and on it: L = 16, 128 walkers in launches of
+// their own, 10^4 trials each, 83.3 and 73.5 ms).
+struct ThreadParams {
+    int L, N, nwalk, W, wM, walker0;
+    long long tstride;
+    uint32_t key0, key1, divL, pad;
+    const int4 *rect;
+    const int32_t *active;
+    uint32_t *spins;
+    int32_t *we, *wm;
+    unsigned long long *wt;
+    DevState *st;
+    double *lng;
+    float2 *lng2;
+    float *lng1;
+    int32_t *H;
+    float *scr;
+};
+
 template <int WPR, int PREC, bool REG>
-__global__ void __launch_bounds__(128) k_sweep_thread(Params p, unsigned long long ntrials)
+__global__ void __launch_bounds__(128) k_sweep_thread(ThreadParams p, unsigned long long ntrials)
 {
     after_previous();
     using TB = Tab<PREC>;
@@ -335,12 +358,14 @@ cudaError_t launch_thread(const Params &p, int blocks, int wpb, uint64_t ntrials
 {
     const bool reg = p.N <= 64 && p.wpr == 1;
     const size_t smem = reg ? 0 : (size_t)p.nwords * wpb * sizeof(uint32_t);
+    const ThreadParams q = {p.L, p.N, p.nwalk, p.W, p.wM, p.walker0, p.tstride, p.key0, p.key1, p.divL, 0, p.rect, p.active,
+                            p.spins, p.we, p.wm, p.wt, p.st, p.lng, p.lng2, p.lng1, p.H, p.scr};
     auto go = [&](auto kern) -> cudaError_t {
         if (smem > 48 * 1024) {
             const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kern<<<blocks, wpb, smem, s>>>(p, (unsigned long long)ntrials);
+        kern<<<blocks, wpb, smem, s>>>(q, (unsigned long long)ntrials);
         return cudaGetLastError();
     };
 #define REWL_THREAD_P(P_)                                              \
