@@ -742,18 +742,21 @@ __device__ __forceinline__ unsigned long long lng_bits(typename Tab<PREC>::Elem 
 }
 
 // Bounded by HBM (8 + 4 bytes an entry) and, beside it, by the 64-bit integer
-// work of the three mixes.  A block takes DIGEST_CHUNK entries of one walker,
-// four adjacent ones a thread at a time: no division per entry, 16-byte loads.
-// L = 64, 4096 walkers (34 GB), f32x2: 27.6 -> 8.5 ms (a grid-stride loop with a
-// 64-bit division per entry before, every value formed in FP64).
-constexpr int DIGEST_CHUNK = 8192;
+// work of the three mixes.  A block takes a chunk of one walker's entries, four
+// adjacent ones a thread at a time: no division per entry, 16-byte loads.  L =
+// 64, 4096 walkers (34 GB), f32x2: 27.6 -> 8.5 ms (a grid-stride loop with a
+// 64-bit division per entry before, every value formed in FP64).  A chunk is
+// 8192 entries where there are many, else down to 1024, so that the SMs share
+// the FP64 work (f32x2, 120 walkers of 7967 bins, all visited: 41 us a call at
+// 8192, 29 at 1024).
+constexpr int DIGEST_CHUNK = 8192, DIGEST_CHUNK_MIN = 1024;
 
 template <int PREC, bool SMALL>     // SMALL: fewer than 2^32 entries
-__global__ void __launch_bounds__(256) k_digest(Params p, int chunks, unsigned long long *out)
+__global__ void __launch_bounds__(256) k_digest(Params p, int chunk, int chunks, unsigned long long *out)
 {
     using Elem = typename Tab<PREC>::Elem;
     const size_t w = blockIdx.x / (unsigned)chunks;
-    const int b0 = (int)(blockIdx.x % (unsigned)chunks) * DIGEST_CHUNK, b1 = min(p.T, b0 + DIGEST_CHUNK);
+    const int b0 = (int)(blockIdx.x % (unsigned)chunks) * chunk, b1 = min(p.T, b0 + chunk);
     const double lnf = p.st->lnf;
     const Elem *B = reinterpret_cast<const Elem *>(PREC == REWL_FP64 ? (const void *)p.lng
                                                  : PREC == REWL_F32X2 ? (const void *)p.lng2 : (const void *)p.lng1)
@@ -791,9 +794,11 @@ __global__ void __launch_bounds__(256) k_digest(Params p, int chunks, unsigned l
 
 cudaError_t launch_digest(const Params &p, unsigned long long *d_out, cudaStream_t s)
 {
-    const int chunks = (p.T + DIGEST_CHUNK - 1) / DIGEST_CHUNK;
-    const unsigned blocks = (unsigned)p.nwalk * (unsigned)chunks;
-    auto go = [&](auto kern) { kern<<<blocks, 256, 0, s>>>(p, chunks, d_out); };
+    int chunk = DIGEST_CHUNK;
+    auto chunks = [&] { return (p.T + chunk - 1) / chunk; };
+    while (chunk > DIGEST_CHUNK_MIN && (long long)p.nwalk * chunks() < 152 * 16) chunk /= 2;
+    const unsigned blocks = (unsigned)p.nwalk * (unsigned)chunks();
+    auto go = [&](auto kern) { kern<<<blocks, 256, 0, s>>>(p, chunk, chunks(), d_out); };
     const bool small = (unsigned long long)p.nwalk * (unsigned long long)p.T < 1ull << 32;
     if (p.precision == REWL_FP64) small ? go(k_digest<REWL_FP64, true>) : go(k_digest<REWL_FP64, false>);
     else if (p.precision == REWL_F32X2) small ? go(k_digest<REWL_F32X2, true>) : go(k_digest<REWL_F32X2, false>);
