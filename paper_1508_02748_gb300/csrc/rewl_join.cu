@@ -60,43 +60,45 @@ __device__ __forceinline__ double warp_sum(double v)
 
 // Sums of exp(v - top) find the top, the largest value, by integers (an FP64
 // comparison occupies its pipe like an addition does): the bits of a double,
-// the negative ones' flipped but for the sign, order like the value.  All 64 of
-// them count: a top that misses the largest value by a part in 2^20 lets exp
-// overflow from ln g = 2^30 on, and cuts all terms off below -2^26.
+// the negative ones' flipped but for the sign, order like the value, and a
+// value's rank is how far it lies below +infinity in that order.  All 64 bits
+// count: a top that misses the largest value by a part in 2^20 lets exp overflow
+// from ln g = 2^30 on, and cuts all terms off below -2^26.  What is not a number
+// ranks behind -infinity, so that it is never the top.
+typedef unsigned long long Rank;
+constexpr Rank RANK_NONE = 0xFFE0000000000001ull;              // of -infinity
+
 __device__ __forceinline__ int order_of(double v)              // of the upper word alone
 {
     const int h = __double2hiint(v);
     return h ^ ((h >> 31) & 0x7FFFFFFF);
 }
 
-constexpr int ORDER_NONE = (int)0xFFF00000 ^ 0x7FFFFFFF;       // of -infinity
-constexpr long long KEY_NONE = (long long)ORDER_NONE * (1ll << 32) + 0xFFFFFFFFll;
-
-__device__ __forceinline__ long long key_of(double v)
+__device__ __forceinline__ Rank rank_of(double v)
 {
-    const unsigned sign = (unsigned)(__double2hiint(v) >> 31);
-    return (long long)(((unsigned long long)(unsigned)order_of(v) << 32) | ((unsigned)__double2loint(v) ^ sign));
+    const unsigned lo = (unsigned)__double2loint(v) ^ (unsigned)(__double2hiint(v) >> 31);
+    return 0x7FF0000000000000ull - ((Rank)(unsigned)order_of(v) << 32 | lo);
 }
 
-__device__ __forceinline__ double value_of(long long key)
+__device__ __forceinline__ double value_of(Rank r)
 {
-    const int h = (int)(key >> 32);
-    return __hiloint2double(h ^ ((h >> 31) & 0x7FFFFFFF), (int)((unsigned)key ^ (unsigned)(h >> 31)));
+    const Rank k = 0x7FF0000000000000ull - r;
+    const int h = (int)(k >> 32);
+    return __hiloint2double(h ^ ((h >> 31) & 0x7FFFFFFF), (int)((unsigned)k ^ (unsigned)(h >> 31)));
 }
 
-__device__ __forceinline__ long long warp_max_key(long long k)
+__device__ __forceinline__ Rank warp_first(Rank r)
 {
-    const int h = (int)(k >> 32), m = __reduce_max_sync(0xFFFFFFFFu, h);
-    const unsigned l = __reduce_max_sync(0xFFFFFFFFu, h == m ? (unsigned)k : 0u);
-    return (long long)(((unsigned long long)(unsigned)m << 32) | l);
+    const unsigned h = (unsigned)(r >> 32), m = __reduce_min_sync(0xFFFFFFFFu, h);
+    return (Rank)m << 32 | __reduce_min_sync(0xFFFFFFFFu, h == m ? (unsigned)r : 0xFFFFFFFFu);
 }
 
 // The upper words tell which terms are certainly LSE_FAR below the top, `far`
-// the order of top - LSE_FAR; what is not a number counts as a term (the
-// negative ones order below -infinity).
+// the order of top - LSE_FAR; what is not a number counts as a term.
 __device__ __forceinline__ bool counts(double v, int far)
 {
-    return (unsigned)order_of(v) - (unsigned)ORDER_NONE >= (unsigned)far - (unsigned)ORDER_NONE;
+    constexpr unsigned none = 0xFFF00000u ^ 0x7FFFFFFFu;       // of -infinity
+    return (unsigned)order_of(v) - none >= (unsigned)far - none;
 }
 
 // ln sum_i exp(v[i]) over the finite v[0..n) by one warp: the top, then the
@@ -104,11 +106,11 @@ __device__ __forceinline__ bool counts(double v, int far)
 __device__ __forceinline__ double lse_warp(const double *v, int n)
 {
     const int lane = threadIdx.x & 31;
-    long long key = KEY_NONE;
-    for (int i = lane; i < n; i += 32) key = max(key, key_of(v[i]));
-    key = warp_max_key(key);
-    if (key == KEY_NONE) return -INFINITY;
-    const double top = value_of(key);
+    Rank first = RANK_NONE;
+    for (int i = lane; i < n; i += 32) first = min(first, rank_of(v[i]));
+    first = warp_first(first);
+    if (first == RANK_NONE) return -INFINITY;
+    const double top = value_of(first);
     const int far = order_of(top - LSE_FAR);
     double acc = 0.0;
     for (int i = lane; i < n; i += 32) {
@@ -168,7 +170,10 @@ __device__ int match_point_block(const double *Ga, const double *Gb, int lo, int
         if (!some(a0) || !some(a1) || !some(b0) || !some(b1)) continue;
         const double ba = (a1 - a0) * inv_step;
         const double bb = (b1 - b0) * inv_step;
-        const long long d = __double_as_longlong(fabs(ba - bb));
+        // (the sign by an integer operation: fabs may make the bits of what is not
+        // a number negative, and so the smallest)
+        const double x = ba - bb;
+        const long long d = (long long)(__double2hiint(x) & 0x7FFFFFFF) << 32 | (unsigned)__double2loint(x);
         if (d < bestd) { bestd = d; best = q; }
     }
     block_min_pair(bestd, best, s_d, s_q);
@@ -524,19 +529,26 @@ __global__ void __launch_bounds__(ROW_COLS * ROW_ES) k_marg_row(Params p, JoinSc
             const double *col = j.piece + (size_t)A * p.tstride + (m - R0.z);
             const int e0 = p.rect[A].x;
             const double c = p.join_rule == 1 && to > from ? j.eslice[(size_t)A * p.wM + (m - R0.z)] : j.eshift[A];
-            #pragma unroll 4
-            for (int e = from + ex; e < to; e += ROW_ES) f(col[(size_t)(e - e0) * p.wM] + c);
+            if (isfinite(c)) {
+                #pragma unroll 4
+                for (int e = from + ex; e < to; e += ROW_ES) f(col[(size_t)(e - e0) * p.wM] + c);
+            } else {                               // a bin without a visit stays one
+                for (int e = from + ex; e < to; e += ROW_ES) {
+                    const double v = col[(size_t)(e - e0) * p.wM];
+                    f(some(v) ? v + c : v);
+                }
+            }
         }
     };
-    __shared__ long long s_top[ROW_ES][ROW_COLS];
-    long long key = KEY_NONE;
-    each([&](double v) { key = max(key, key_of(v)); });
-    s_top[ex][cx] = key;
+    __shared__ Rank s_top[ROW_ES][ROW_COLS];
+    Rank first = RANK_NONE;
+    each([&](double v) { first = min(first, rank_of(v)); });
+    s_top[ex][cx] = first;
     __syncthreads();
-    for (int k = 0; k < ROW_ES; ++k) key = max(key, s_top[k][cx]);
-    const double top = value_of(key);
+    for (int k = 0; k < ROW_ES; ++k) first = min(first, s_top[k][cx]);
+    const double top = value_of(first);
     double acc = 0.0;
-    if (key != KEY_NONE) {
+    if (first != RANK_NONE) {
         const int far = order_of(top - LSE_FAR);
         each([&](double v) { if (counts(v, far)) acc += exp(v - top); });
     }
@@ -544,7 +556,7 @@ __global__ void __launch_bounds__(ROW_COLS * ROW_ES) k_marg_row(Params p, JoinSc
     __syncthreads();
     if (ex == 0 && m < B) {
         for (int k = 1; k < ROW_ES; ++k) acc += s_part[k][cx];
-        j.F[(size_t)b * B + m] = key == KEY_NONE ? -INFINITY : top + log(acc);
+        j.F[(size_t)b * B + m] = first == RANK_NONE ? -INFINITY : top + log(acc);
     }
 }
 
@@ -599,15 +611,15 @@ __global__ void __launch_bounds__(MATCH_THREADS) k_match_m(Params p, JoinScratch
     }
 }
 
-// 3c. Assemble the joined table; each block leaves the key of the largest value
+// 3c. Assemble the joined table; each block leaves the rank of the largest value
 // of its part in red[].
-constexpr int RED_BLOCKS = 512;     // red[]: 512 maxima (their keys), then from entry 512 on the sums
+constexpr int RED_BLOCKS = 512;     // red[]: 512 maxima (their ranks), then from entry 512 on the sums
 
 __global__ void __launch_bounds__(256) k_assemble(Params p, JoinScratch j)
 {
     after_previous();
     const int B = p.N + 1;
-    long long key = KEY_NONE;
+    Rank first = RANK_NONE;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < (size_t)B * B; idx += (size_t)gridDim.x * blockDim.x) {
         const int e = (int)(idx / B), m = (int)(idx % B);
         double v = -INFINITY;
@@ -620,40 +632,40 @@ __global__ void __launch_bounds__(256) k_assemble(Params p, JoinScratch j)
             }
         }
         j.J[idx] = v;
-        key = max(key, key_of(v));
+        first = min(first, rank_of(v));
     }
-    key = warp_max_key(key);
-    __shared__ long long s[8];
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = key;
+    first = warp_first(first);
+    __shared__ Rank s[8];
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = first;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < 8; ++k) key = max(key, s[k]);
-        reinterpret_cast<long long *>(j.red)[blockIdx.x] = key;
+        for (int k = 1; k < 8; ++k) first = min(first, s[k]);
+        reinterpret_cast<Rank *>(j.red)[blockIdx.x] = first;
     }
 }
 
 // 4. Normalisation: sums of exp(v - max) by blocks, then the shift that makes
 // sum g = 2^N.  Each block folds the blocks' maxima (sums) itself, all in the
 // same order, instead of waiting for a kernel that does.
-__device__ __forceinline__ long long fold_max(const double *red, int n)
+__device__ __forceinline__ Rank fold_max(const double *red, int n)
 {
-    __shared__ long long s_m[8];
-    long long key = KEY_NONE;
-    for (int k = threadIdx.x; k < n; k += 256) key = max(key, reinterpret_cast<const long long *>(red)[k]);
-    key = warp_max_key(key);
-    if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = key;
+    __shared__ Rank s_m[8];
+    Rank first = RANK_NONE;
+    for (int k = threadIdx.x; k < n; k += 256) first = min(first, reinterpret_cast<const Rank *>(red)[k]);
+    first = warp_first(first);
+    if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = first;
     __syncthreads();
-    for (int k = 0; k < 8; ++k) key = max(key, s_m[k]);
-    return key;
+    for (int k = 0; k < 8; ++k) first = min(first, s_m[k]);
+    return first;
 }
 
 __global__ void __launch_bounds__(256) k_red_sumexp(const double *v, size_t n, double *red, int nblk)
 {
     after_previous();
-    const long long key = fold_max(red, nblk);
-    const double top = value_of(key);
+    const Rank first = fold_max(red, nblk);
+    const double top = value_of(first);
     double acc = 0.0;
-    if (key != KEY_NONE) {
+    if (first != RANK_NONE) {
         const int far = order_of(top - LSE_FAR);
         for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
             const double x = v[i];

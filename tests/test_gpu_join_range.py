@@ -51,6 +51,36 @@ def test_join_of_large_tables(P, offset, nE, nM):
             np.testing.assert_allclose(Jg[fin], Jo[fin], rtol=0, atol=tol)
 
 
+# Tables with entries that are no number or infinite, in one walker or in all:
+# what the oracle's join makes of them, or refuses, this one does too.
+@pytest.mark.parametrize("L,nE,nM,W,seen", [(6, 2, 1, 3, 0.99), (8, 3, 2, 1, 0.9), (12, 4, 1, 3, 0.5), (9, 2, 2, 8, 0.9), (5, 1, 1, 2, 1.0)])
+@pytest.mark.parametrize("bad", [(np.inf, np.inf), (-np.inf, -np.inf), (np.nan, -np.nan), (np.inf, np.nan)])
+def test_join_of_tables_that_are_not_finite(P, L, nE, nM, W, seen, bad):
+    kw = dict(L=L, n_win_E=nE, n_win_M=nM, overlap_E=0.5, overlap_M=0.5, walkers_per_window=W, seed=6, drive_budget=10**8)
+    o, r = OracleREWL(OracleConfig(**kw)), P.REWL(P.Config(**kw))
+    rng = np.random.default_rng(L)
+    for everywhere in (False, True):
+        lng, H = _set(o, [], 11)
+        H = np.where((H >= 0) & (rng.random(H.size) < seen), H, -1).astype(np.int32)
+        n = H.size // (W * nE * nM)
+        for w in range(0, H.size // n, 1 if everywhere else H.size // n):
+            at = w * n + rng.choice(np.flatnonzero(H[w * n:(w + 1) * n] >= 0), 2, replace=False)
+            lng[at] = bad
+        for x in (o, r):
+            x.set_tables(lng, H)
+        for ro, rg in ((oracle.JOIN_MARGINAL, P.JOIN_MARGINAL), (oracle.JOIN_PER_SLICE, P.JOIN_PER_SLICE)):
+            try:
+                Jo, em, mm = o.join(ro)
+            except RuntimeError:
+                with pytest.raises(P.REWLError, match="join failed"):
+                    r.lng(rule=rg)
+                continue
+            Jg, emg, mmg = r.lng(matches=True, rule=rg)
+            np.testing.assert_array_equal(emg, em)
+            np.testing.assert_array_equal(mmg, mm)
+            np.testing.assert_allclose(Jg, Jo, rtol=1e-12, atol=1e-9)
+
+
 def test_join_of_more_windows_than_a_grid_axis(P):
     """257 x 257 windows of 2 x 2 bins cut out of one table, each with an offset
     of its own: joined again, the table comes back up to a constant.  It falls
