@@ -861,7 +861,12 @@ __device__ __forceinline__ double rel_diff(double a, double b)
 }
 
 // Two bins a thread at a time where the three tables allow 16-byte accesses
-// (the last bin of an odd count alone).
+// (the last bin of an odd count alone) and there are enough for all SMs' threads;
+// below that a thread's two tanh in a row are the call's time (4097 bins that
+// differ by more than 1/8: 12.4 us a call with one bin a thread, 15.2 with two;
+// 132,000: 21.2 and 20.5).
+constexpr size_t PAIRS_FROM = 152 * 512;
+
 template <bool PAIRS>
 __global__ void __launch_bounds__(256) k_rel_diff(const double *a, const double *b, double *out, size_t n)
 {
@@ -880,7 +885,7 @@ __global__ void __launch_bounds__(256) k_rel_diff(const double *a, const double 
 cudaError_t launch_rel_diff(const double *a, const double *b, double *out, size_t n, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    const bool pairs = (((uintptr_t)a | (uintptr_t)b | (uintptr_t)out) & 15) == 0;
+    const bool pairs = n >= PAIRS_FROM && (((uintptr_t)a | (uintptr_t)b | (uintptr_t)out) & 15) == 0;
     const size_t want = ((pairs ? (n + 1) / 2 : n) + 255) / 256;
     const int blocks = (int)std::min<size_t>(want, 152 * 16);
     if (pairs) k_rel_diff<true><<<blocks, 256, 0, s>>>(a, b, out, n);

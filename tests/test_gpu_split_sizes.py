@@ -78,3 +78,21 @@ def test_jackknife_of_two_walkers_that_share_no_bin(P):
     mean, err = r.jackknife()
     mo, _ = oracle.jackknife(o)
     assert np.array_equal(mean, np.asarray(mo).reshape(mean.shape)) and np.isneginf(mean).all() and np.isnan(err).all()
+
+
+# Eq. 5 either side of the count from which a thread takes two bins
+@pytest.mark.parametrize("n,shift", [(77_823, 0), (77_824, 0), (77_825, 0), (77_824, 1), (200_001, 0)])
+def test_relative_difference_by_pairs(P, n, shift):
+    import torch
+    rng = np.random.default_rng(n + shift)
+    a = rng.normal(0, 300, n)
+    b = a + np.where(rng.random(n) < 0.5, 1, -1) * 10.0 ** rng.uniform(-13, 2, n)
+    a[rng.integers(0, n, 50)] = -np.inf
+    b[rng.integers(0, n, 50)] = -np.inf
+    a[-1], b[-1] = 0.0, 0.125
+    da, db = (torch.zeros(n + shift, dtype=torch.float64, device="cuda")[shift:].copy_(torch.from_numpy(v)) for v in (a, b))
+    with np.errstate(invalid="ignore"):
+        ref = 2.0 * np.tanh(0.5 * np.abs(a - b))
+    ea, eb = np.isneginf(a), np.isneginf(b)
+    ref = np.where(ea & eb, np.nan, np.where(ea | eb, 2.0, ref))
+    np.testing.assert_allclose(P.relative_difference(da, db).cpu().numpy(), ref, rtol=2e-15, atol=0)
