@@ -70,14 +70,15 @@ extern "C" {
                                    at once and a launch has the trials to pay for it, else global */
 #define REWL_TABLES_GLOBAL 1    /* global memory (L1-cached) */
 #define REWL_TABLES_STAGED 2    /* all of the walker's bins in shared memory for the launch (REWL_E_CUDA
-                                   at launch when they do not fit) */
+                                   at launch when they do not fit; where they do, but not with the
+                                   entries kept around them, global) */
 
 /* How the warp sampler holds a walker's lattice during a launch
  * (rewl_config.lattice_mode); every choice gives the same trajectory. */
 #define REWL_LATTICE_AUTO 0     /* a register when N <= 64 and the tables are staged or a walker has 8
                                    lanes, else shared memory */
 #define REWL_LATTICE_REGISTER 1 /* one 64-bit register per lane (N <= 64 only, else REWL_E_INVALID) */
-#define REWL_LATTICE_SHARED 2   /* one 32-bit word per row in shared memory (two for L > 32) */
+#define REWL_LATTICE_SHARED 2   /* 32-bit words in shared memory, one to three a row */
 
 /* Sampling kernels (same trajectory, different mapping onto the GPU). */
 #define REWL_SAMPLER_WARP 0     /* 8/16/32 lanes per walker, 3/4/5 trials resolved per step */

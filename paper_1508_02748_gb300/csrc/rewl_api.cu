@@ -313,16 +313,16 @@ int max_pairs_of(const Dims &d)
 // what the configuration fixes stays.  Every choice gives the same chains.
 // Times are ms per 10^4 trials of every walker on a GB300.
 //   - Staged tables while all walkers fit on the GPU's shared memory at once:
-//     L = 8, 3 x 3 windows, staged against global: 36 walkers 0.36 / 0.55, 1350
-//     0.60 / 0.81; past that the staged walkers take turns (1800: 0.97 with 16
-//     lanes, global 0.82).
+//     L = 8, 3 x 3 windows, staged against global: 36 walkers 0.33 / 0.55, 1350
+//     0.62 / 0.78; past that the staged walkers take turns (1800: 0.94 with 16
+//     lanes, global 0.80).
 //   - And while the launch pays for the staging, some 1.4 ns a bin against 10
 //     ns a trial (20 with a register lattice): from a trial for 12 (16) bins on.
 //     One window, us a cycle staged / global: L = 12 (21,025 bins) 48 / 21 at
 //     100 trials, 85 / 74 at 1000, 172 / 185 at 3000; L = 10 (10,201) 39 / 30 at
 //     300, 68 / 71 at 1000; L = 8 (4225) 21 / 17 at 100, 27 / 30 at 300.
-//   - Staged: 32 lanes up to two warps per SM sub-partition (900 walkers 0.47,
-//     16 lanes 0.49), then 16 (1350: 0.62 against 0.60); more walkers make the
+//   - Staged: 32 lanes up to two warps per SM sub-partition (900 walkers 0.48,
+//     16 lanes 0.47), then 16 (1350: 0.66 against 0.62); more walkers make the
 //     step's instructions count, fewer its depth.
 //   - Global: 32 lanes while that is at most the 18 warps an SM that the
 //     registers allow (L = 32, 2048 walkers 1.03, 16 lanes 1.19; 2560: 1.16 and

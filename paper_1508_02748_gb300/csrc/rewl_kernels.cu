@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(256) k_flat(Params p)
 
 cudaError_t launch_flat(const Params &p, cudaStream_t s)
 {
-    // blocks a walker: until 8 blocks an SM or until a block has 8192 bins
+    // blocks a walker: up to 8, while there are fewer than 4 an SM and each has 8192 bins
     int parts = 1;
     while (parts < 8 && (long long)p.nwalk * parts < 152 * 4 && p.T / (2 * parts) >= 8192) parts *= 2;
     if (parts == 1) {

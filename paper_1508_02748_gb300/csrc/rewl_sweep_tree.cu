@@ -75,7 +75,7 @@
 // comparisons, the leaf by shuffle instead of a mailbox, the trial read a step
 // ahead and near-ties looked at on the path alone took 266-302 instructions a
 // step to 149-157.  Sampling launches of 10^4 trials per walker, GB300, 2070
-// MHz, before -> after: L = 8 (36 walkers, 32 lanes, staged) 0.72 -> 0.35 ms; L
+// MHz, before -> after: L = 8 (36 walkers, 32 lanes, staged) 0.72 -> 0.34 ms; L
 // = 16 (256 walkers, 32 lanes) 0.95 -> 0.63 ms; L = 32 (2048 walkers, 32 lanes)
 // 1.64 -> 1.03 ms; L = 64 (3904 walkers, 16 lanes) 2.71 -> 1.56 ms.
 // Tried and slower: the visits of recent bins in a shared-memory cache (L1
@@ -239,9 +239,9 @@ __global__ void __launch_bounds__(256) k_sweep_tree(Params p, unsigned ntrials, 
     // Staging in and out of a window by one warp: the entries come by copies
     // that no register waits for, their addresses by a walk through the rows
     // (loads, stores and a division an entry before: 3.4 ns a bin in and out, 1.4
-    // so; L = 8's 64 cycles 23.2 -> 22.4 ms).  Windows of at most 26 x 26 bins
-    // (N <= 32) keep the short form: they have little to stage, and the step
-    // compiled with the walk took 2% longer there.
+    // so; L = 8, 36 walkers, 64 cycles 23.2 -> 22.4 ms).  Windows of at most 26 x
+    // 26 bins (N <= 32) keep the short form: they have little to stage, and the
+    // step compiled with the walk took 2% longer there.
     constexpr bool WALK = SMT && LAT != 1;
     auto each_bin = [&](auto f) {                   // f(bin, its entry), every G-th one
         const int by = G / wM;                      // rows that G bins are on
